@@ -41,20 +41,14 @@
 #include <cmath>
 #include <vector>
 
-#include "mfmc_internal.h"
-#include "smem_fft.cuh"
-#include "trace.cuh"
+#include "active_set_tile.cuh"
 
 namespace mfmc {
 
 constexpr int AS_NT = 512;
-constexpr float AS_CG_RTOL = 1e-5f;   // max |J d + F| / max |F| that ends a correction
 constexpr int AS_VEC64 = 3;           // u, g, w
 constexpr int AS_VEC32 = 7;           // d, r, p, q, inactive mask, z, t
 constexpr int AS_MAX_LEVELS = 8;
-constexpr int AS_NU = 2;              // damped-Jacobi sweeps before and after each coarse correction
-constexpr int AS_NU_COARSE = 16;
-constexpr float AS_OMEGA = 0.8f;
 constexpr int AS_SPECTRAL_MIN_DISC = 100;  // disc points from which the disc sum is spectral
 
 // Multigrid levels of the CG preconditioner: n_0 = n, halved while even and >= 16 (the coarsest
@@ -351,12 +345,7 @@ __global__ void __launch_bounds__(AS_NT) active_set_kernel(ActiveSetArgs a) {
         else if (a.own_fft) {  // (the coarse levels in shared memory hold nothing between steps)
             auto ld = [&](int y, int x) { return U[y * n + x]; };
             auto put = [&](int y, int x, double S) { G[y * n + x] = e2a * S + a.cF * U[y * n + x]; };
-            switch (n) {  // the paper's meshes on compile-time plans
-                case 64: cta_disc_sums<64, double>(a.plan, as_smem, a.khat, a.tw, ld, put); break;
-                case 88: cta_disc_sums<88, double>(a.plan, as_smem, a.khat, a.tw, ld, put); break;
-                case 128: cta_disc_sums<128, double>(a.plan, as_smem, a.khat, a.tw, ld, put); break;
-                default: cta_disc_sums<0, double>(a.plan, as_smem, a.khat, a.tw, ld, put); break;
-            }
+            cta_disc_sums<0, double>(a.plan, as_smem, a.khat, a.tw, ld, put);
         } else as_for(n, [&](int y, int x, int i) {
             double S = 0.0;
             for (int dy = -R; dy <= R; ++dy) {
@@ -497,7 +486,9 @@ mfmc_status run_solve_active_set(Model &m, const double *eps_dev, const float *u
                                  float *uT, double *ubar, double *ooi, cudaStream_t st) {
     if (!(m.d.beta2 > 0.0)) return fail(MFMC_EINVAL, "the active-set solver is for beta2 > 0");
     if (ns == 0) return MFMC_OK;
-    const size_t per = as_per_sample(m.d.n);
+    // n = 64, 88, 128 (the paper's lattices): the correction solve on chip; other n: the kernel above
+    const bool tile = as_tile_supported(m.d.n);
+    const size_t per = tile ? as_tile_per_sample(m.d.n) : as_per_sample(m.d.n);
     mfmc_status s = grow_buffer(&m.as_buf, &m.as_cap, ns * per);
     if (s != MFMC_OK) return s;
     if (!m.d_status) {
@@ -511,7 +502,7 @@ mfmc_status run_solve_active_set(Model &m, const double *eps_dev, const float *u
     if (!m.d_as_iters) MFMC_CUDA(cudaMalloc((void **)&m.d_as_iters, 2 * sizeof(unsigned long long)));
     MFMC_CUDA(cudaMemsetAsync(m.d_as_iters, 0, 2 * sizeof(unsigned long long), st));
     // the inactive-set vector starts at an impossible value, so no step sees a stale set
-    MFMC_CUDA(cudaMemsetAsync(m.as_buf, 0xff, ns * per * sizeof(double), st));
+    if (!tile) MFMC_CUDA(cudaMemsetAsync(m.as_buf, 0xff, ns * per * sizeof(double), st));
     ActiveSetArgs a;
     a.u0 = u0;
     a.uT = uT;
@@ -563,6 +554,41 @@ mfmc_status run_solve_active_set(Model &m, const double *eps_dev, const float *u
         a.khat = m.d_khat64;
         a.tw = m.d_tw64;
         smem = std::max(smem, fft_smem_bytes<double>(n, AS_NT / 32));
+    }
+    if (tile) {
+        AsTileArgs t{};
+        t.u0 = u0;
+        t.uT = uT;
+        t.ubar = ubar;
+        t.ooi = ooi;
+        t.eps = eps_dev;
+        t.eps_nominal = a.eps_nominal;
+        t.buf = a.buf;
+        t.status = a.status;
+        t.iters = a.iters;
+        t.wtab = a.wtab;
+        for (int d = 0; d <= kMaxR; ++d) t.widths[d] = a.widths[d];
+        t.R = a.R;
+        t.nsteps = nsteps;
+        t.newton_max = a.newton_max;
+        t.cg_max = a.cg_max;
+        t.own_fft = a.own_fft;
+        t.plan = a.plan;
+        t.khat = a.khat;
+        t.tw = a.tw;
+        t.trace = a.trace;
+        t.ahat = a.ahat;
+        t.chat = a.chat;
+        t.tau = a.tau;
+        t.beta1 = a.beta1;
+        t.beta2 = a.beta2;
+        t.cF = a.cF;
+        for (size_t o = 0; o < ns; o += 65535) {
+            t.s0 = o;
+            s = launch_active_set_tile(t, m.d.n, (unsigned)std::min<size_t>(65535, ns - o), st);
+            if (s != MFMC_OK) return s;
+        }
+        return MFMC_OK;
     }
     MFMC_CUDA(cudaFuncSetAttribute(active_set_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     auto launch = [&](int load, int steps, int g_given, int finish) -> mfmc_status {

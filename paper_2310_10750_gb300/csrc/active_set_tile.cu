@@ -1,0 +1,705 @@
+// The beta2 > 0 step (MFMC_ALGO_ACTIVE_SET) on n = 64, 88 and 128: the method of active_set.cu,
+// one CTA per sample, with the FP32 correction solve held in registers and shared memory.
+//
+// Layout.  Warp w owns lattice rows 8w .. 8w + 7 and a lane 2 or 4 consecutive columns of them
+// (n = 64: 2 columns, 32 lanes, 8 warps; n = 88: 4 columns, 22 lanes, 11 warps; n = 128: 4
+// columns, 32 lanes, 16 warps), so a row is one warp, its periodic wrap a shuffle, and only a
+// warp's first and last row pass through shared memory when a stencil is applied.  The residual
+// of the correction (f) and the V-cycle's iterate (v) are registers; p and q are shared memory,
+// each thread reading back its own values; d is global scratch that is only added to (a vector
+// reduction, no load).  The inactive set is one bit per point, a 32-bit mask per thread.
+//
+// The multigrid levels halve the thread's block: 4 x 8, 2 x 4 and 1 x 2 points (n = 64: 2 x 8
+// and 1 x 4), each level's mask average a population count of the thread's bits, restriction
+// and prolongation exchanging one row per warp.  The levels below one column a lane (16^2 and
+// 8^2, or 11^2 for n = 88) are a warp's work in shared memory.  A pass costs one CTA barrier (the
+// row exchange alternates two buffers), no division and no index arithmetic.
+//
+// What bounds it: the fallback kernel (fine-level vectors in L2, generic indices) issued 943
+// instructions per point and CG iteration, and waited on L2 (long scoreboard 4.4 cycles an
+// instruction).  Here the FP64 pipe (two lanes a clock an SM) takes the larger part of a step:
+// the disc sum's transforms and 8 operations per point of a Newton residual.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+
+#include "active_set_tile.cuh"
+
+namespace mfmc {
+
+namespace {
+
+template <int N>
+struct AtCfg {
+    static constexpr int CW = N == 64 ? 2 : 4;      // columns per lane
+    static constexpr int LU = N / CW;               // lanes in use
+    static constexpr int RW = 8;                    // rows per warp
+    static constexpr int NW = N / RW, NT = 32 * NW;
+    static constexpr int LEVELS = CW == 4 ? 3 : 2;  // levels held in registers: CW >> level columns a lane
+    static constexpr int TN = N >> LEVELS;          // the first level of the one-warp part
+    static constexpr int TN2 = TN % 2 == 0 && TN >= 16 ? TN / 2 : 0;  // its second level, if any
+    static constexpr int XP = 32 * CW;              // floats of an exchanged row
+    // shared memory (floats): p, q, the exchange rows (two buffers of two rows a warp), then per
+    // one-warp level v, r, f, omega / diagonal, diagonal
+    static constexpr int P = 0, Q = N * N, X = 2 * N * N, T = X + 4 * NW * XP;
+    static constexpr int T2 = T + 5 * TN * TN;
+    static constexpr size_t SMEM = (size_t)(T2 + 5 * TN2 * TN2) * sizeof(float);
+    static_assert(LU <= 32 && N % RW == 0 && N % CW == 0, "one warp per row block");
+};
+
+__device__ __forceinline__ double at_clip(double v) { return v > 1.0 ? 1.0 : (v < -1.0 ? -1.0 : v); }
+
+template <int C>
+__device__ __forceinline__ void at_ld(float (&v)[C], const float *p) {
+    if constexpr (C == 4) {
+        const float4 t = *reinterpret_cast<const float4 *>(p);
+        v[0] = t.x, v[1] = t.y, v[2] = t.z, v[3] = t.w;
+    } else if constexpr (C == 2) {
+        const float2 t = *reinterpret_cast<const float2 *>(p);
+        v[0] = t.x, v[1] = t.y;
+    } else {
+        v[0] = *p;
+    }
+}
+template <int C>
+__device__ __forceinline__ void at_st(float *p, const float (&v)[C]) {
+    if constexpr (C == 4)
+        *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    else if constexpr (C == 2)
+        *reinterpret_cast<float2 *>(p) = make_float2(v[0], v[1]);
+    else
+        *p = v[0];
+}
+template <int C>
+__device__ __forceinline__ void at_ld64(double (&v)[C], const double *p) {
+#pragma unroll
+    for (int c = 0; c < C; c += 2) {
+        const double2 t = *reinterpret_cast<const double2 *>(p + c);
+        v[c] = t.x, v[c + 1] = t.y;
+    }
+}
+template <int C>
+__device__ __forceinline__ void at_st64(double *p, const double (&v)[C]) {
+#pragma unroll
+    for (int c = 0; c < C; c += 2) *reinterpret_cast<double2 *>(p + c) = make_double2(v[c], v[c + 1]);
+}
+// d += v at C consecutive floats of global memory that only this thread touches (no load; the
+// values are read back past L1).
+template <int C>
+__device__ __forceinline__ void at_red(float *p, const float (&v)[C]) {
+    if constexpr (C == 4)
+        asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3])
+                     : "memory");
+    else
+        asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(v[0]), "f"(v[1]) : "memory");
+}
+
+// A thread's view of the CTA and the operator.  Level l: J v = (tb1 + 4 tb2[l] + m icg) v - tb2[l] (sum
+// of the four neighbours), m the mean of the inactive set over the level's 2^l x 2^l points.
+template <int N>
+struct At {
+    using K = AtCfg<N>;
+    float *sm, *red;
+    int warp, lane, left, right;  // lanes of the columns left and right of the lane's (periodic)
+    int par, rpar;                // the exchange and reduction buffers in turn
+    unsigned mask;                // inactive set: bit row * CW + column
+    float tb1, icg, tb2;          // tb2: level 0; level l has tb2 / 4^l
+
+    __device__ __forceinline__ float *xrow(int w, int which) const {
+        return sm + K::X + ((par * K::NW + w) * 2 + which) * K::XP;
+    }
+    __device__ __forceinline__ int up() const { return warp == 0 ? K::NW - 1 : warp - 1; }
+    __device__ __forceinline__ int down() const { return warp == K::NW - 1 ? 0 : warp + 1; }
+    // Rows next to the warp's: the last row of the warp above and the first of the warp below.
+    template <int C>
+    __device__ __forceinline__ void exchange(const float (&top)[C], const float (&bot)[C], float (&above)[C],
+                                             float (&below)[C]) {
+        at_st<C>(xrow(warp, 0) + lane * C, top);
+        at_st<C>(xrow(warp, 1) + lane * C, bot);
+        __syncthreads();
+        at_ld<C>(above, xrow(up(), 1) + lane * C);
+        at_ld<C>(below, xrow(down(), 0) + lane * C);
+        par ^= 1;
+    }
+    template <int C>
+    __device__ __forceinline__ void from_above(const float (&bot)[C], float (&above)[C]) {
+        at_st<C>(xrow(warp, 1) + lane * C, bot);
+        __syncthreads();
+        at_ld<C>(above, xrow(up(), 1) + lane * C);
+        par ^= 1;
+    }
+    template <int C>
+    __device__ __forceinline__ void from_below(const float (&top)[C], float (&below)[C]) {
+        at_st<C>(xrow(warp, 0) + lane * C, top);
+        __syncthreads();
+        at_ld<C>(below, xrow(down(), 0) + lane * C);
+        par ^= 1;
+    }
+    // CTA-wide sum in a fixed order: butterflies over the lanes, then over the warps' sums (the
+    // same in every warp).  Idle lanes pass 0.
+    __device__ __forceinline__ float sum(float v) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) red[rpar * 32 + warp] = v;
+        __syncthreads();
+        float t = lane < K::NW ? red[rpar * 32 + lane] : 0.f;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        rpar ^= 1;
+        return t;
+    }
+    // CTA-wide maximum of non-negative values (their bit patterns order as unsigned integers).
+    __device__ __forceinline__ float max(float v) {
+        const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(v));
+        if (lane == 0) red[rpar * 32 + warp] = __uint_as_float(m);
+        __syncthreads();
+        const unsigned t = __reduce_max_sync(0xffffffffu, lane < K::NW ? __float_as_uint(red[rpar * 32 + lane]) : 0u);
+        rpar ^= 1;
+        return __uint_as_float(t);
+    }
+
+    template <int L>
+    __device__ __forceinline__ float tb2l() const { return tb2 * (1.0f / (1 << (2 * L))); }
+    template <int L>
+    __host__ __device__ static constexpr unsigned bits(int y, int c) {
+        unsigned b = 0;
+        for (int i = 0; i < (1 << L); ++i)
+            for (int j = 0; j < (1 << L); ++j) b |= 1u << (((y << L) + i) * K::CW + (c << L) + j);
+        return b;
+    }
+    // The diagonal of J at the lane's point (y, c) of level L.
+    template <int L>
+    __device__ __forceinline__ float diag(int y, int c) const {
+        const float d = tb1 + 4.0f * tb2l<L>();
+        if constexpr (L == 0)
+            return (mask & bits<0>(y, c)) ? d + icg : d;
+        else
+            return fmaf((float)__popc(mask & bits<L>(y, c)), icg * (1.0f / (1 << (2 * L))), d);
+    }
+    template <int L>
+    __device__ __forceinline__ float relax(int y, int c) const {  // omega / diagonal
+        const float d = tb1 + 4.0f * tb2l<L>();
+        if constexpr (L == 0)
+            return (mask & bits<0>(y, c)) ? __fdividef(AS_OMEGA, d + icg) : __fdividef(AS_OMEGA, d);
+        else
+            return __fdividef(AS_OMEGA, diag<L>(y, c));
+    }
+};
+
+// One row's neighbour sums: up + down + left + right.
+template <int N, int C>
+__device__ __forceinline__ void at_nb(const At<N> &t, const float (&up)[C], const float (&cur)[C], const float (&dn)[C],
+                                      float (&S)[C]) {
+    const float l = __shfl_sync(0xffffffffu, cur[C - 1], t.left), r = __shfl_sync(0xffffffffu, cur[0], t.right);
+#pragma unroll
+    for (int c = 0; c < C; ++c) S[c] = (up[c] + dn[c]) + ((c == 0 ? l : cur[c - 1]) + (c == C - 1 ? r : cur[c + 1]));
+}
+
+// One damped-Jacobi sweep of v in place: v + omega D^-1 (f - J v) = (1 - omega) v + omega D^-1 (f + tb2 S).
+template <int N, int L, int C, int R>
+__device__ __forceinline__ void at_sweep(At<N> &t, const float (&f)[R][C], float (&v)[R][C]) {
+    float prev[C], below[C];
+    t.template exchange<C>(v[0], v[R - 1], prev, below);
+    const float tb2 = t.template tb2l<L>();
+#pragma unroll
+    for (int y = 0; y < R; ++y) {
+        float S[C];
+        at_nb<N, C>(t, prev, v[y], y == R - 1 ? below : v[y + 1 < R ? y + 1 : y], S);
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            prev[c] = v[y][c];
+            v[y][c] = fmaf(t.template relax<L>(y, c), fmaf(tb2, S[c], f[y][c]), (1.0f - AS_OMEGA) * v[y][c]);
+        }
+    }
+}
+
+// The horizontally weighted residual rows h (weights 1 2 1 over 4, at every second column) of
+// v against f, for the full-weighting restriction.
+template <int N, int L, int C, int R>
+__device__ __forceinline__ void at_residual_rows(At<N> &t, const float (&f)[R][C], float (&v)[R][C],
+                                                 float (&h)[R][C > 1 ? C / 2 : 1]) {
+    float prev[C], below[C];
+    t.template exchange<C>(v[0], v[R - 1], prev, below);
+    const float tb2 = t.template tb2l<L>();
+#pragma unroll
+    for (int y = 0; y < R; ++y) {
+        float S[C], r[C];
+        at_nb<N, C>(t, prev, v[y], y == R - 1 ? below : v[y + 1 < R ? y + 1 : y], S);
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            prev[c] = v[y][c];
+            r[c] = fmaf(-t.template diag<L>(y, c), v[y][c], fmaf(tb2, S[c], f[y][c]));
+        }
+        const float l = __shfl_sync(0xffffffffu, r[C - 1], t.left);
+        if constexpr (C > 1) {
+#pragma unroll
+            for (int X = 0; X < C / 2; ++X) h[y][X] = 0.25f * ((X == 0 ? l : r[2 * X - 1]) + r[2 * X + 1]) + 0.5f * r[2 * X];
+        } else {
+            const float rr = __shfl_sync(0xffffffffu, r[0], t.right);
+            h[y][0] = 0.25f * (l + rr) + 0.5f * r[0];
+        }
+    }
+}
+
+// ------------------------------------------------------------------- the one-warp levels
+// Arrays of a level of n x n: v, r, f, w = omega / diagonal, d = diagonal.
+template <int n>
+struct TailLvl {
+    float *v, *r, *f, *w, *d;
+    __device__ explicit TailLvl(float *b) : v(b), r(b + n * n), f(b + 2 * n * n), w(b + 3 * n * n), d(b + 4 * n * n) {}
+};
+
+template <int n, typename Fn>
+__device__ __forceinline__ void tail_for(int lane, Fn fn) {
+#pragma unroll
+    for (int i0 = 0; i0 < n * n; i0 += 32) {
+        const int i = i0 + lane;
+        if (n * n % 32 == 0 || i < n * n) fn(i / n, i % n, i);
+    }
+}
+
+template <int n>
+__device__ __forceinline__ float tail_nb(const float *v, int y, int x) {
+    const int ym = y == 0 ? n - 1 : y - 1, yp = y == n - 1 ? 0 : y + 1;
+    const int xm = x == 0 ? n - 1 : x - 1, xp = x == n - 1 ? 0 : x + 1;
+    return (v[ym * n + x] + v[yp * n + x]) + (v[y * n + xm] + v[y * n + xp]);
+}
+
+template <int n>
+__device__ __forceinline__ void tail_sweep(const TailLvl<n> &T, const float *src, float *dst, float tb2, int lane) {
+    tail_for<n>(lane, [&](int y, int x, int i) {
+        dst[i] = fmaf(T.w[i], fmaf(tb2, tail_nb<n>(src, y, x), T.f[i]), (1.0f - AS_OMEGA) * src[i]);
+    });
+    __syncwarp();
+}
+
+template <int n>
+__device__ __forceinline__ void tail_zero_sweep(const TailLvl<n> &T, float *dst, int lane) {
+    tail_for<n>(lane, [&](int, int, int i) { dst[i] = T.w[i] * T.f[i]; });
+    __syncwarp();
+}
+
+template <int n>
+__device__ __forceinline__ void tail_coarsest(const TailLvl<n> &T, float tb2, int lane) {
+    tail_zero_sweep<n>(T, T.r, lane);
+#pragma unroll 1
+    for (int k = 2; k <= AS_NU_COARSE; k += 2) {
+        tail_sweep<n>(T, T.r, T.v, tb2, lane);
+        if (k < AS_NU_COARSE) tail_sweep<n>(T, T.v, T.r, tb2, lane);
+    }
+}
+
+// One cycle from f to v on the one-warp levels, n and (n2 > 0) n2 = n / 2.
+template <int n, int n2>
+__device__ __forceinline__ void tail_cycle(float *base, float tb2, int lane) {
+    const TailLvl<n> T(base);
+    if constexpr (n2 == 0) {
+        tail_coarsest<n>(T, tb2, lane);
+    } else {
+        const TailLvl<n2> B(base + 5 * n * n);
+        tail_zero_sweep<n>(T, T.r, lane);
+        tail_sweep<n>(T, T.r, T.v, tb2, lane);
+        tail_for<n>(lane, [&](int y, int x, int i) {
+            T.r[i] = fmaf(-T.d[i], T.v[i], fmaf(tb2, tail_nb<n>(T.v, y, x), T.f[i]));
+        });
+        __syncwarp();
+        tail_for<n2>(lane, [&](int Y, int X, int i) {  // full weighting at (2Y, 2X)
+            const int y = 2 * Y, x = 2 * X, ym = y == 0 ? n - 1 : y - 1, xm = x == 0 ? n - 1 : x - 1;
+            const float *r = T.r;
+            const float k = (r[ym * n + xm] + r[ym * n + x + 1]) + (r[(y + 1) * n + xm] + r[(y + 1) * n + x + 1]);
+            B.f[i] = (4.0f * r[y * n + x] + 2.0f * tail_nb<n>(r, y, x) + k) * 0.0625f;
+        });
+        __syncwarp();
+        tail_coarsest<n2>(B, 0.25f * tb2, lane);
+        tail_for<n>(lane, [&](int y, int x, int i) {
+            const int Y = y >> 1, X = x >> 1;
+            const int Y1 = (y & 1) ? (Y + 1 == n2 ? 0 : Y + 1) : Y, X1 = (x & 1) ? (X + 1 == n2 ? 0 : X + 1) : X;
+            T.v[i] += 0.25f * ((B.v[Y * n2 + X] + B.v[Y * n2 + X1]) + (B.v[Y1 * n2 + X] + B.v[Y1 * n2 + X1]));
+        });
+        __syncwarp();
+        tail_sweep<n>(T, T.v, T.r, tb2, lane);
+        tail_sweep<n>(T, T.r, T.v, tb2, lane);
+    }
+}
+
+// ------------------------------------------------------------------------- the register levels
+// v = B f on level L and below: two damped-Jacobi sweeps (the first from zero), the coarse
+// correction (full weighting, bilinear prolongation), two sweeps.
+template <int N, int L, int C, int R>
+__device__ __forceinline__ void at_cycle(At<N> &t, const float (&f)[R][C], float (&v)[R][C]) {
+    using K = AtCfg<N>;
+#pragma unroll
+    for (int y = 0; y < R; ++y)
+#pragma unroll
+        for (int c = 0; c < C; ++c) v[y][c] = t.template relax<L>(y, c) * f[y][c];
+    at_sweep<N, L, C, R>(t, f, v);
+    constexpr int HC = C > 1 ? C / 2 : 1;
+    float cf[R / 2][HC];
+    {
+        float h[R][HC], ha[HC];
+        at_residual_rows<N, L, C, R>(t, f, v, h);
+        t.template from_above<HC>(h[R - 1], ha);
+#pragma unroll
+        for (int Y = 0; Y < R / 2; ++Y)
+#pragma unroll
+            for (int X = 0; X < HC; ++X)
+                cf[Y][X] = 0.25f * ((Y == 0 ? ha[X] : h[Y == 0 ? 0 : 2 * Y - 1][X]) + h[2 * Y + 1][X]) + 0.5f * h[2 * Y][X];
+    }
+    if constexpr (C > 1) {
+        float e[R / 2][HC], eb[HC], er[R / 2 + 1];
+        at_cycle<N, L + 1, HC, R / 2>(t, cf, e);
+        t.template from_below<HC>(e[0], eb);
+#pragma unroll
+        for (int Y = 0; Y < R / 2; ++Y) er[Y] = __shfl_sync(0xffffffffu, e[Y][0], t.right);
+        er[R / 2] = __shfl_sync(0xffffffffu, eb[0], t.right);
+#pragma unroll
+        for (int Y = 0; Y < R / 2; ++Y) {
+            float a[HC + 1], b[HC + 1];  // coarse rows Y and Y + 1 with the column to the right
+#pragma unroll
+            for (int X = 0; X < HC; ++X) {
+                a[X] = e[Y][X];
+                b[X] = Y + 1 < R / 2 ? e[Y + 1 < R / 2 ? Y + 1 : Y][X] : eb[X];
+            }
+            a[HC] = er[Y];
+            b[HC] = er[Y + 1];
+#pragma unroll
+            for (int X = 0; X < HC; ++X) {
+                const float m0 = 0.5f * (a[X] + a[X + 1]), m1 = 0.5f * (b[X] + b[X + 1]);
+                v[2 * Y][2 * X] += a[X];
+                v[2 * Y][2 * X + 1] += m0;
+                v[2 * Y + 1][2 * X] += 0.5f * (a[X] + b[X]);
+                v[2 * Y + 1][2 * X + 1] += 0.5f * (m0 + m1);
+            }
+        }
+    } else {
+        constexpr int TN = K::TN;
+        const TailLvl<TN> T(t.sm + K::T);
+        if ((t.lane & 1) == 0 && t.lane < K::LU) {
+#pragma unroll
+            for (int Y = 0; Y < R / 2; ++Y) T.f[(t.warp * (R / 2) + Y) * TN + (t.lane >> 1)] = cf[Y][0];
+        }
+        __syncthreads();
+        if (t.warp == 0) tail_cycle<TN, K::TN2>(t.sm + K::T, t.template tb2l<L + 1>(), t.lane);
+        __syncthreads();
+        const int x = t.lane < K::LU ? t.lane : 0, X = x >> 1, X1 = (x & 1) ? (X + 1 == TN ? 0 : X + 1) : X;
+#pragma unroll
+        for (int y = 0; y < R; ++y) {
+            const int Y = t.warp * (R / 2) + (y >> 1), Y1 = (y & 1) ? (Y + 1 == TN ? 0 : Y + 1) : Y;
+            v[y][0] += 0.25f * ((T.v[Y * TN + X] + T.v[Y * TN + X1]) + (T.v[Y1 * TN + X] + T.v[Y1 * TN + X1]));
+        }
+    }
+    at_sweep<N, L, C, R>(t, f, v);
+    at_sweep<N, L, C, R>(t, f, v);
+}
+
+// Diagonals of the one-warp levels from the threads' masks: the count over a 2^LEVELS square is
+// the lane's block of 2^LEVELS rows and the right lane's.
+template <int N>
+__device__ __forceinline__ void at_tail_diagonals(At<N> &t) {
+    using K = AtCfg<N>;
+    constexpr int TN = K::TN, LV = K::LEVELS, TR = K::RW >> LV;
+    constexpr float area = 1.0f / (1 << (2 * LV));
+    const TailLvl<TN> T(t.sm + K::T);
+    const float tb2 = t.tb2 * area, d0 = t.tb1 + 4.0f * tb2;
+#pragma unroll
+    for (int Y = 0; Y < TR; ++Y) {
+        const unsigned rows = t.mask & ((K::CW << LV) == 32 ? 0xffffffffu
+                                                            : ((1u << ((K::CW << LV) & 31)) - 1u) << (Y * (K::CW << LV)));
+        const int own = __popc(rows), both = own + __shfl_sync(0xffffffffu, own, t.right);
+        if ((t.lane & 1) == 0 && t.lane < K::LU) {
+            const int i = (t.warp * TR + Y) * TN + (t.lane >> 1);
+            T.d[i] = fmaf((float)both, t.icg * area, d0);
+            T.w[i] = __fdividef(AS_OMEGA, T.d[i]);
+        }
+    }
+    if constexpr (K::TN2 > 0) {
+        __syncthreads();
+        if (t.warp == 0) {
+            constexpr int n2 = K::TN2;
+            const TailLvl<n2> B(t.sm + K::T2);
+            const float e0 = t.tb1 + tb2;  // 4 (tb2 / 4)
+            tail_for<n2>(t.lane, [&](int Y, int X, int i) {
+                const float *d = T.d + 2 * Y * TN + 2 * X;
+                const float m = 0.25f * ((d[0] + d[1]) + (d[TN] + d[TN + 1])) - d0;  // mean of m icg
+                B.d[i] = e0 + m;
+                B.w[i] = __fdividef(AS_OMEGA, B.d[i]);
+            });
+        }
+    }
+}
+
+template <int N, int MINB>
+__global__ void __launch_bounds__(AtCfg<N>::NT, MINB) active_set_tile_kernel(const __grid_constant__ AsTileArgs a) {
+    using K = AtCfg<N>;
+    constexpr int CW = K::CW, RW = K::RW, nn = N * N;
+    extern __shared__ __align__(16) float at_smem[];
+    __shared__ float red[64];
+    __shared__ int widths[kMaxR + 1];
+    __shared__ double red64[K::NW];
+    const size_t smp = a.s0 + blockIdx.x;
+    const unsigned long long t_start = a.trace.rec ? trace_clock() : 0ull;
+    At<N> t;
+    t.sm = at_smem;
+    t.red = red;
+    t.warp = threadIdx.x >> 5;
+    t.lane = threadIdx.x & 31;
+    const bool act = t.lane < K::LU;
+    t.left = t.lane == 0 ? K::LU - 1 : t.lane - 1;
+    t.right = t.lane >= K::LU - 1 ? 0 : t.lane + 1;
+    t.par = t.rpar = 0;
+    t.mask = 0u;
+    double *U = a.buf + smp * as_tile_per_sample(N), *G = U + nn, *W = G + nn;
+    // the thread's slot of p, q and d: row y at + y * N * NW floats... [row][warp][lane] vectors
+    const int slot = (t.warp * K::LU + t.lane) * CW;
+    constexpr int SROW = K::NW * K::LU * CW;
+    float *D = reinterpret_cast<float *>(W + nn) + slot, *Pp = at_smem + K::P + slot, *Qp = at_smem + K::Q + slot;
+    const int own = t.warp * RW * N + (act ? t.lane : 0) * CW;  // the thread's first point
+    if (threadIdx.x <= a.R) widths[threadIdx.x] = a.widths[threadIdx.x];
+    const double eps = a.eps ? a.eps[smp] : a.eps_nominal;
+    const double e2a = eps * eps * a.ahat, cg = e2a * a.chat, icg = 1.0 / cg;
+    const double tb1 = a.tau * a.beta1, tb2h = a.tau * a.beta2 * (double)N * (double)N;
+    const double wdiag = tb1 + 4.0 * tb2h;
+    t.tb1 = (float)tb1;
+    t.icg = (float)icg;
+    t.tb2 = (float)tb2h;
+    for (int i = threadIdx.x; i < nn; i += K::NT) U[i] = (double)a.u0[smp * (size_t)nn + i];
+    __syncthreads();
+    bool failed = false;
+    unsigned long long n_newton = 0, n_cg = 0;
+    for (int step = 1; step <= a.nsteps && !failed; ++step) {
+        // explicit part g = gamma * u + c_F u
+        if (a.own_fft) {
+            cta_disc_sums<N, double>(
+                a.plan, at_smem, a.khat, a.tw, [&](int y, int x) { return U[y * N + x]; },
+                [&](int y, int x, double S) { G[y * N + x] = e2a * S + a.cF * U[y * N + x]; });
+        } else {
+            for (int i = threadIdx.x; i < nn; i += K::NT) {
+                const int y = i / N, x = i - y * N;
+                double S = 0.0;
+                for (int dy = -a.R; dy <= a.R; ++dy) {
+                    const int ady = dy < 0 ? -dy : dy, w = widths[ady];
+                    int yy = y + dy;
+                    yy += yy < 0 ? N : 0;
+                    yy -= yy >= N ? N : 0;
+                    int xx = x - w;
+                    xx += xx < 0 ? N : 0;
+                    for (int dx = -w; dx <= w; ++dx) {
+                        S += a.wtab ? a.wtab[ady * ady + dx * dx] * U[yy * N + xx] : U[yy * N + xx];
+                        xx = xx == N - 1 ? 0 : xx + 1;
+                    }
+                }
+                G[i] = e2a * S + a.cF * U[i];
+            }
+            __syncthreads();
+        }
+        if (step == 1) {  // start: w of the previous step, or here the beta2 = 0 step's
+            for (int i = threadIdx.x; i < nn; i += K::NT) {
+                const double u0 = at_clip((U[i] + tb1 * G[i]) / (1.0 + tb1 * cg));
+                W[i] = cg * u0 - G[i];
+            }
+            __syncthreads();
+        }
+        for (int it = 1;; ++it) {
+            ++n_newton;
+            // FP64 residual F(w), the inactive set, and the right-hand side f = -F of J d = -F
+            float f[RW][CW];
+            float fmax = 0.0f;
+            unsigned now = 0u;
+            {
+                double up[CW], cur[CW], dn[CW];
+                at_ld64<CW>(up, W + (t.warp == 0 ? nn - N + own : own - N));
+                at_ld64<CW>(cur, W + own);
+#pragma unroll
+                for (int y = 0; y < RW; ++y) {
+                    const int i = own + y * N;
+                    double g[CW], u[CW];
+                    at_ld64<CW>(dn, W + (y == RW - 1 && t.warp == K::NW - 1 ? i + N - nn : i + N));
+                    at_ld64<CW>(g, G + i);
+                    at_ld64<CW>(u, U + i);
+                    const double l = __shfl_sync(0xffffffffu, cur[CW - 1], t.left);
+                    const double r = __shfl_sync(0xffffffffu, cur[0], t.right);
+#pragma unroll
+                    for (int c = 0; c < CW; ++c) {
+                        const double S = (up[c] + dn[c]) + ((c == 0 ? l : cur[c > 0 ? c - 1 : 0]) +
+                                                            (c == CW - 1 ? r : cur[c + 1 < CW ? c + 1 : c]));
+                        const double xv = (cur[c] + g[c]) * icg;
+                        // |x| < 1 and the projection from the exponent bits (no FP64 compares)
+                        const int hi = __double2hiint(xv);
+                        const bool in = (hi & 0x7fffffff) < 0x3ff00000;
+                        const double xc = in ? xv : __hiloint2double((hi & 0x80000000) | 0x3ff00000, 0);
+                        const double F = fma(wdiag, cur[c], fma(-tb2h, S, xc - u[c]));
+                        now |= in ? 1u << (y * CW + c) : 0u;
+                        f[y][c] = act ? -(float)F : 0.0f;
+                        fmax = fmaxf(fmax, fabsf(f[y][c]));
+                    }
+#pragma unroll
+                    for (int c = 0; c < CW; ++c) {
+                        up[c] = cur[c];
+                        cur[c] = dn[c];
+                    }
+                }
+            }
+            const bool changed = __syncthreads_or(act && now != t.mask);
+            t.mask = now;
+            fmax = t.max(fmax);
+            if (it > 1 && !changed && fmax <= 1e-11f) break;
+            if (it > a.newton_max) {
+                failed = true;
+                break;
+            }
+            if (fmax == 0.0f) continue;  // F = 0 with a new active set: the next pass confirms it
+            at_tail_diagonals<N>(t);
+            const float sc = 1.0f / fmax;  // scaled to max |f| = 1
+#pragma unroll
+            for (int y = 0; y < RW; ++y)
+#pragma unroll
+                for (int c = 0; c < CW; ++c) f[y][c] *= sc;
+            // CG on J d = f from d = 0, preconditioned by one V-cycle
+            float rz = 0.0f;
+            for (int k = 1;; ++k) {
+                float v[RW][CW];
+                at_cycle<N, 0, CW, RW>(t, f, v);
+                float dot = 0.0f;
+#pragma unroll
+                for (int y = 0; y < RW; ++y)
+#pragma unroll
+                    for (int c = 0; c < CW; ++c) dot = fmaf(f[y][c], v[y][c], dot);
+                const float rz2 = t.sum(act ? dot : 0.0f), beta = k == 1 ? 0.0f : rz2 / rz;
+                rz = rz2;
+                // p = z + beta p, q = J z + beta q
+                float pq = 0.0f;
+                {
+                    float prev[CW], below[CW];
+                    t.template exchange<CW>(v[0], v[RW - 1], prev, below);
+#pragma unroll
+                    for (int y = 0; y < RW; ++y) {
+                        float S[CW], p[CW], q[CW];
+                        at_nb<N, CW>(t, prev, v[y], y == RW - 1 ? below : v[y + 1 < RW ? y + 1 : y], S);
+                        if (k > 1 && act) {
+                            at_ld<CW>(p, Pp + y * SROW);
+                            at_ld<CW>(q, Qp + y * SROW);
+                        } else {
+#pragma unroll
+                            for (int c = 0; c < CW; ++c) p[c] = q[c] = 0.0f;
+                        }
+#pragma unroll
+                        for (int c = 0; c < CW; ++c) {
+                            prev[c] = v[y][c];
+                            const float jz = fmaf(t.template diag<0>(y, c), v[y][c], -t.tb2 * S[c]);
+                            p[c] = fmaf(beta, p[c], v[y][c]);
+                            q[c] = fmaf(beta, q[c], jz);
+                            pq = fmaf(p[c], q[c], pq);
+                        }
+                        if (act) {
+                            at_st<CW>(Pp + y * SROW, p);
+                            at_st<CW>(Qp + y * SROW, q);
+                        }
+                    }
+                }
+                pq = t.sum(act ? pq : 0.0f);
+                const float alpha = pq > 0.0f ? rz / pq : 0.0f;
+                float rmax = 0.0f;
+                if (act) {
+#pragma unroll
+                    for (int y = 0; y < RW; ++y) {
+                        float p[CW], q[CW];
+                        at_ld<CW>(p, Pp + y * SROW);
+                        at_ld<CW>(q, Qp + y * SROW);
+#pragma unroll
+                        for (int c = 0; c < CW; ++c) {
+                            p[c] *= alpha;
+                            f[y][c] = fmaf(-alpha, q[c], f[y][c]);
+                            rmax = fmaxf(rmax, fabsf(f[y][c]));
+                        }
+                        if (k == 1)
+                            at_st<CW>(D + y * SROW, p);
+                        else
+                            at_red<CW>(D + y * SROW, p);
+                    }
+                }
+                rmax = t.max(rmax);
+                if (rmax <= AS_CG_RTOL || !(pq > 0.0f) || !(rz > 0.0f) || k >= a.cg_max) {
+                    n_cg += k;
+                    break;
+                }
+            }
+            if (act) {
+                const double scale = (double)fmax;
+#pragma unroll
+                for (int y = 0; y < RW; ++y) {
+                    double w[CW];
+                    at_ld64<CW>(w, W + own + y * N);
+#pragma unroll
+                    for (int c = 0; c < CW; ++c) w[c] = fma(scale, (double)__ldcg(D + y * SROW + c), w[c]);
+                    at_st64<CW>(W + own + y * N, w);
+                }
+            }
+            __syncthreads();
+        }
+        if (failed) break;
+        if (act) {
+#pragma unroll
+            for (int y = 0; y < RW; ++y) {
+                double w[CW], g[CW];
+                at_ld64<CW>(w, W + own + y * N);
+                at_ld64<CW>(g, G + own + y * N);
+#pragma unroll
+                for (int c = 0; c < CW; ++c) w[c] = at_clip((w[c] + g[c]) * icg);
+                at_st64<CW>(U + own + y * N, w);
+            }
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        atomicAdd(&a.iters[0], n_newton);
+        atomicAdd(&a.iters[1], n_cg);
+        trace_put(a.trace, kTraceActiveSet, (uint32_t)smp, (uint32_t)a.nsteps, t_start);
+    }
+    if (failed) {
+        if (threadIdx.x == 0) atomicExch(a.status, 1);
+        return;
+    }
+    double s = 0.0;
+    for (int i = threadIdx.x; i < nn; i += K::NT) {
+        const double u = U[i];
+        s += u;
+        if (a.uT) a.uT[smp * (size_t)nn + i] = (float)u;
+    }
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (t.lane == 0) red64[t.warp] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double tot = 0.0;
+        for (int i = 0; i < K::NW; ++i) tot += red64[i];
+        const double mean = tot / (double)nn;
+        if (a.ubar) a.ubar[smp] = mean;
+        if (a.ooi) a.ooi[smp] = 0.5 * (1.0 + mean);
+    }
+}
+
+template <int N, int MINB>
+mfmc_status at_launch(const AsTileArgs &a, unsigned grid, cudaStream_t st) {
+    using K = AtCfg<N>;
+    size_t smem = K::SMEM;
+    if (a.own_fft) smem = std::max(smem, fft_smem_bytes<double>(N, K::NW));
+    auto kern = active_set_tile_kernel<N, MINB>;
+    MFMC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kern<<<grid, K::NT, smem, st>>>(a);
+    MFMC_LAUNCHED("active_set_tile launch");
+    return MFMC_OK;
+}
+
+}  // namespace
+
+bool as_tile_supported(int n) { return n == 64 || n == 88 || n == 128; }
+
+mfmc_status launch_active_set_tile(const AsTileArgs &a, int n, unsigned grid, cudaStream_t st) {
+    switch (n) {
+        case 64: return at_launch<64, 3>(a, grid, st);
+        case 88: return at_launch<88, 1>(a, grid, st);
+        case 128: return at_launch<128, 1>(a, grid, st);
+        default: return fail(MFMC_EINVAL, "no on-chip active-set kernel for n = %d", n);
+    }
+}
+
+}  // namespace mfmc
