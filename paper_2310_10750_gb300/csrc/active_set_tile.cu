@@ -12,7 +12,7 @@
 // The multigrid levels halve the thread's block: 4 x 8, 2 x 4 and 1 x 2 points (n = 64: 2 x 8
 // and 1 x 4), each level's mask average a population count of the thread's bits, restriction
 // and prolongation exchanging one row per warp.  The levels below one column a lane (16^2 and
-// 8^2, or 11^2 for n = 88) are a warp's work in shared memory.  A pass costs one CTA barrier (the
+// 8^2, or 11^2 for n = 88) are one warp's work, in its registers.  A pass costs one CTA barrier (the
 // row exchange alternates two buffers), no division and no index arithmetic.
 //
 // What bounds it: the fallback kernel (fine-level vectors in L2, generic indices) issued 943
@@ -37,13 +37,11 @@ struct AtCfg {
     static constexpr int NW = N / RW, NT = 32 * NW;
     static constexpr int LEVELS = CW == 4 ? 3 : 2;  // levels held in registers: CW >> level columns a lane
     static constexpr int TN = N >> LEVELS;          // the first level of the one-warp part
-    static constexpr int TN2 = TN % 2 == 0 && TN >= 16 ? TN / 2 : 0;  // its second level, if any
     static constexpr int XP = 32 * CW;              // floats of an exchanged row
-    // shared memory (floats): p, q, the exchange rows (two buffers of two rows a warp), then per
-    // one-warp level v, r, f, omega / diagonal, diagonal
+    // shared memory (floats): p, q, the exchange rows (two buffers of two rows a warp), then the
+    // one-warp part's right-hand side, diagonal and result
     static constexpr int P = 0, Q = N * N, X = 2 * N * N, T = X + 4 * NW * XP;
-    static constexpr int T2 = T + 5 * TN * TN;
-    static constexpr size_t SMEM = (size_t)(T2 + 5 * TN2 * TN2) * sizeof(float);
+    static constexpr size_t SMEM = (size_t)(T + 3 * TN * TN) * sizeof(float);
     static_assert(LU <= 32 && N % RW == 0 && N % CW == 0, "one warp per row block");
 };
 
@@ -104,6 +102,7 @@ struct At {
     int par, rpar;                // the exchange and reduction buffers in turn
     unsigned mask;                // inactive set: bit row * CW + column
     float tb1, icg, tb2;          // tb2: level 0; level l has tb2 / 4^l
+    float w0, w1, d0, d1;         // level 0: omega / diagonal and diagonal off and on the inactive set
 
     __device__ __forceinline__ float *xrow(int w, int which) const {
         return sm + K::X + ((par * K::NW + w) * 2 + which) * K::XP;
@@ -172,15 +171,14 @@ struct At {
     __device__ __forceinline__ float diag(int y, int c) const {
         const float d = tb1 + 4.0f * tb2l<L>();
         if constexpr (L == 0)
-            return (mask & bits<0>(y, c)) ? d + icg : d;
+            return (mask & bits<0>(y, c)) ? d1 : d0;
         else
             return fmaf((float)__popc(mask & bits<L>(y, c)), icg * (1.0f / (1 << (2 * L))), d);
     }
     template <int L>
     __device__ __forceinline__ float relax(int y, int c) const {  // omega / diagonal
-        const float d = tb1 + 4.0f * tb2l<L>();
         if constexpr (L == 0)
-            return (mask & bits<0>(y, c)) ? __fdividef(AS_OMEGA, d + icg) : __fdividef(AS_OMEGA, d);
+            return (mask & bits<0>(y, c)) ? w1 : w0;
         else
             return __fdividef(AS_OMEGA, diag<L>(y, c));
     }
@@ -242,83 +240,131 @@ __device__ __forceinline__ void at_residual_rows(At<N> &t, const float (&f)[R][C
 }
 
 // ------------------------------------------------------------------- the one-warp levels
-// Arrays of a level of n x n: v, r, f, w = omega / diagonal, d = diagonal.
+// A level of n x n (n = 16, 8 or 11) in one warp's registers: lane g n + x holds column x of the rows
+// g R .. g R + R - 1 (G row groups, n = G R; lanes from G n on are idle and mirror lane 0).
 template <int n>
-struct TailLvl {
-    float *v, *r, *f, *w, *d;
-    __device__ explicit TailLvl(float *b) : v(b), r(b + n * n), f(b + 2 * n * n), w(b + 3 * n * n), d(b + 4 * n * n) {}
+struct TailCfg {
+    static constexpr int G = n == 16 ? 2 : (n == 8 ? 4 : 1), R = n / G;
+    static_assert(G * n <= 32 && G * R == n, "one warp");
+};
+template <int n>
+struct TailLanes {
+    int g, x, left, right, above, below;  // the lane's place and the lanes of its neighbours
+    __device__ explicit TailLanes(int lane) {
+        using T = TailCfg<n>;
+        const int l = lane < T::G * n ? lane : 0;
+        g = l / n;
+        x = l - g * n;
+        left = l + (x == 0 ? n - 1 : -1);
+        right = l + (x == n - 1 ? 1 - n : 1);
+        above = (g == 0 ? T::G - 1 : g - 1) * n + x;
+        below = (g == T::G - 1 ? 0 : g + 1) * n + x;
+    }
 };
 
-template <int n, typename Fn>
-__device__ __forceinline__ void tail_for(int lane, Fn fn) {
+__device__ __forceinline__ float tail_shfl(float v, int lane) { return __shfl_sync(0xffffffffu, v, lane); }
+
+// The neighbour sums of every point of the lane.
+template <int n>
+__device__ __forceinline__ void tail_nb(const TailLanes<n> &p, const float (&v)[TailCfg<n>::R], float (&S)[TailCfg<n>::R]) {
+    constexpr int R = TailCfg<n>::R;
+    const float a = TailCfg<n>::G == 1 ? v[R - 1] : tail_shfl(v[R - 1], p.above);
+    const float b = TailCfg<n>::G == 1 ? v[0] : tail_shfl(v[0], p.below);
 #pragma unroll
-    for (int i0 = 0; i0 < n * n; i0 += 32) {
-        const int i = i0 + lane;
-        if (n * n % 32 == 0 || i < n * n) fn(i / n, i % n, i);
+    for (int y = 0; y < R; ++y)
+        S[y] = ((y == 0 ? a : v[y > 0 ? y - 1 : 0]) + (y == R - 1 ? b : v[y + 1 < R ? y + 1 : y])) +
+               (tail_shfl(v[y], p.left) + tail_shfl(v[y], p.right));
+}
+
+// One damped-Jacobi sweep in place: w = omega / diagonal.
+template <int n>
+__device__ __forceinline__ void tail_sweep(const TailLanes<n> &p, const float (&f)[TailCfg<n>::R],
+                                           const float (&w)[TailCfg<n>::R], float (&v)[TailCfg<n>::R], float tb2) {
+    float S[TailCfg<n>::R];
+    tail_nb<n>(p, v, S);
+#pragma unroll
+    for (int y = 0; y < TailCfg<n>::R; ++y) v[y] = fmaf(w[y], fmaf(tb2, S[y], f[y]), (1.0f - AS_OMEGA) * v[y]);
+}
+
+template <int n>
+__device__ __forceinline__ void tail_coarsest(const TailLanes<n> &p, const float (&f)[TailCfg<n>::R],
+                                              const float (&d)[TailCfg<n>::R], float (&v)[TailCfg<n>::R], float tb2) {
+    float w[TailCfg<n>::R];
+#pragma unroll
+    for (int y = 0; y < TailCfg<n>::R; ++y) {
+        w[y] = __fdividef(AS_OMEGA, d[y]);
+        v[y] = w[y] * f[y];
     }
-}
-
-template <int n>
-__device__ __forceinline__ float tail_nb(const float *v, int y, int x) {
-    const int ym = y == 0 ? n - 1 : y - 1, yp = y == n - 1 ? 0 : y + 1;
-    const int xm = x == 0 ? n - 1 : x - 1, xp = x == n - 1 ? 0 : x + 1;
-    return (v[ym * n + x] + v[yp * n + x]) + (v[y * n + xm] + v[y * n + xp]);
-}
-
-template <int n>
-__device__ __forceinline__ void tail_sweep(const TailLvl<n> &T, const float *src, float *dst, float tb2, int lane) {
-    tail_for<n>(lane, [&](int y, int x, int i) {
-        dst[i] = fmaf(T.w[i], fmaf(tb2, tail_nb<n>(src, y, x), T.f[i]), (1.0f - AS_OMEGA) * src[i]);
-    });
-    __syncwarp();
-}
-
-template <int n>
-__device__ __forceinline__ void tail_zero_sweep(const TailLvl<n> &T, float *dst, int lane) {
-    tail_for<n>(lane, [&](int, int, int i) { dst[i] = T.w[i] * T.f[i]; });
-    __syncwarp();
-}
-
-template <int n>
-__device__ __forceinline__ void tail_coarsest(const TailLvl<n> &T, float tb2, int lane) {
-    tail_zero_sweep<n>(T, T.r, lane);
 #pragma unroll 1
-    for (int k = 2; k <= AS_NU_COARSE; k += 2) {
-        tail_sweep<n>(T, T.r, T.v, tb2, lane);
-        if (k < AS_NU_COARSE) tail_sweep<n>(T, T.v, T.r, tb2, lane);
-    }
+    for (int k = 2; k <= AS_NU_COARSE; ++k) tail_sweep<n>(p, f, w, v, tb2);
 }
 
-// One cycle from f to v on the one-warp levels, n and (n2 > 0) n2 = n / 2.
-template <int n, int n2>
-__device__ __forceinline__ void tail_cycle(float *base, float tb2, int lane) {
-    const TailLvl<n> T(base);
-    if constexpr (n2 == 0) {
-        tail_coarsest<n>(T, tb2, lane);
-    } else {
-        const TailLvl<n2> B(base + 5 * n * n);
-        tail_zero_sweep<n>(T, T.r, lane);
-        tail_sweep<n>(T, T.r, T.v, tb2, lane);
-        tail_for<n>(lane, [&](int y, int x, int i) {
-            T.r[i] = fmaf(-T.d[i], T.v[i], fmaf(tb2, tail_nb<n>(T.v, y, x), T.f[i]));
-        });
-        __syncwarp();
-        tail_for<n2>(lane, [&](int Y, int X, int i) {  // full weighting at (2Y, 2X)
-            const int y = 2 * Y, x = 2 * X, ym = y == 0 ? n - 1 : y - 1, xm = x == 0 ? n - 1 : x - 1;
-            const float *r = T.r;
-            const float k = (r[ym * n + xm] + r[ym * n + x + 1]) + (r[(y + 1) * n + xm] + r[(y + 1) * n + x + 1]);
-            B.f[i] = (4.0f * r[y * n + x] + 2.0f * tail_nb<n>(r, y, x) + k) * 0.0625f;
-        });
-        __syncwarp();
-        tail_coarsest<n2>(B, 0.25f * tb2, lane);
-        tail_for<n>(lane, [&](int y, int x, int i) {
-            const int Y = y >> 1, X = x >> 1;
-            const int Y1 = (y & 1) ? (Y + 1 == n2 ? 0 : Y + 1) : Y, X1 = (x & 1) ? (X + 1 == n2 ? 0 : X + 1) : X;
-            T.v[i] += 0.25f * ((B.v[Y * n2 + X] + B.v[Y * n2 + X1]) + (B.v[Y1 * n2 + X] + B.v[Y1 * n2 + X1]));
-        });
-        __syncwarp();
-        tail_sweep<n>(T, T.v, T.r, tb2, lane);
-        tail_sweep<n>(T, T.r, T.v, tb2, lane);
+// One cycle from f to v (shared memory, n x n) by one warp; d: the diagonals.
+template <int n>
+__device__ __noinline__ void tail_cycle(const float *fs, const float *ds, float *vs, float tb1, float tb2, int lane) {
+    constexpr int R = TailCfg<n>::R, G = TailCfg<n>::G;
+    const TailLanes<n> p(lane);
+    float f[R], d[R], v[R];
+#pragma unroll
+    for (int y = 0; y < R; ++y) {
+        f[y] = fs[(p.g * R + y) * n + p.x];
+        d[y] = ds[(p.g * R + y) * n + p.x];
+    }
+    if constexpr (n != 16) {
+        tail_coarsest<n>(p, f, d, v, tb2);
+    } else {  // 16^2 over 8^2: lane 16 g + x of 16^2 holds rows 8 g .., lane 8 g + x of 8^2 rows 2 g, 2 g + 1
+        const TailLanes<8> q(lane);
+        float w[R], S[R], h[R], fc[2], dc[2], vc[2];
+#pragma unroll
+        for (int y = 0; y < R; ++y) {
+            w[y] = __fdividef(AS_OMEGA, d[y]);
+            v[y] = w[y] * f[y];
+        }
+        tail_sweep<n>(p, f, w, v, tb2);
+        tail_nb<n>(p, v, S);
+#pragma unroll
+        for (int y = 0; y < R; ++y) {  // residual, weighted 1 2 1 along x
+            const float r = fmaf(-d[y], v[y], fmaf(tb2, S[y], f[y]));
+            h[y] = 0.25f * (tail_shfl(r, p.left) + tail_shfl(r, p.right)) + 0.5f * r;
+        }
+        const float ha = tail_shfl(h[R - 1], p.above);
+        // coarse rows 4 g' .. of this lane's column (g' = its half), then to the 8^2 owners; the coarse
+        // mean of m icg is the diagonals' mean less the stencil's part
+        float cf[R / 2], cd[R / 2];
+        const float s16 = tb1 + 4.0f * tb2, s8 = tb1 + tb2;
+#pragma unroll
+        for (int Y = 0; Y < R / 2; ++Y) {
+            cf[Y] = 0.25f * ((Y == 0 ? ha : h[Y > 0 ? 2 * Y - 1 : 0]) + h[2 * Y + 1]) + 0.5f * h[2 * Y];
+            const float dd = d[2 * Y] + d[2 * Y + 1];
+            cd[Y] = 0.25f * (dd + tail_shfl(dd, p.right)) - s16 + s8;
+        }
+        const int from = (q.g >> 1) * 16 + 2 * q.x;  // rows 2 q.g, 2 q.g + 1 = rows 2 (q.g & 1), + 1 of that half
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const float f0 = tail_shfl(cf[i], from), f1 = tail_shfl(cf[2 + i], from);
+            const float d0 = tail_shfl(cd[i], from), d1 = tail_shfl(cd[2 + i], from);
+            fc[i] = (q.g & 1) ? f1 : f0;
+            dc[i] = (q.g & 1) ? d1 : d0;
+        }
+        tail_coarsest<8>(q, fc, dc, vc, 0.25f * tb2);
+        // bilinear prolongation: coarse rows 4 g .. 4 g + 4 at columns x / 2 and (x odd) the next
+        float e[R / 2 + 1];
+        const int X = p.x >> 1, X1 = (p.x & 1) ? ((X + 1) & 7) : X;
+#pragma unroll
+        for (int Y = 0; Y <= R / 2; ++Y) {
+            const int yc = (4 * p.g + Y) & 7, base = (yc >> 1) * 8;
+            const float a0 = tail_shfl(vc[0], base + X), a1 = tail_shfl(vc[1], base + X);
+            const float b0 = tail_shfl(vc[0], base + X1), b1 = tail_shfl(vc[1], base + X1);
+            e[Y] = 0.5f * ((Y & 1) ? a1 + b1 : a0 + b0);  // 4 g is even: the row's parity is Y's
+        }
+#pragma unroll
+        for (int y = 0; y < R; ++y) v[y] += (y & 1) ? 0.5f * (e[y >> 1] + e[(y >> 1) + 1]) : e[y >> 1];
+        tail_sweep<n>(p, f, w, v, tb2);
+        tail_sweep<n>(p, f, w, v, tb2);
+    }
+    if (lane < G * n) {
+#pragma unroll
+        for (int y = 0; y < R; ++y) vs[(p.g * R + y) * n + p.x] = v[y];
     }
 }
 
@@ -373,57 +419,41 @@ __device__ __forceinline__ void at_cycle(At<N> &t, const float (&f)[R][C], float
         }
     } else {
         constexpr int TN = K::TN;
-        const TailLvl<TN> T(t.sm + K::T);
+        float *tf = t.sm + K::T, *td = tf + TN * TN, *tv = td + TN * TN;
         if ((t.lane & 1) == 0 && t.lane < K::LU) {
 #pragma unroll
-            for (int Y = 0; Y < R / 2; ++Y) T.f[(t.warp * (R / 2) + Y) * TN + (t.lane >> 1)] = cf[Y][0];
+            for (int Y = 0; Y < R / 2; ++Y) tf[(t.warp * (R / 2) + Y) * TN + (t.lane >> 1)] = cf[Y][0];
         }
         __syncthreads();
-        if (t.warp == 0) tail_cycle<TN, K::TN2>(t.sm + K::T, t.template tb2l<L + 1>(), t.lane);
+        if (t.warp == 0) tail_cycle<TN>(tf, td, tv, t.tb1, t.template tb2l<L + 1>(), t.lane);
         __syncthreads();
         const int x = t.lane < K::LU ? t.lane : 0, X = x >> 1, X1 = (x & 1) ? (X + 1 == TN ? 0 : X + 1) : X;
 #pragma unroll
         for (int y = 0; y < R; ++y) {
             const int Y = t.warp * (R / 2) + (y >> 1), Y1 = (y & 1) ? (Y + 1 == TN ? 0 : Y + 1) : Y;
-            v[y][0] += 0.25f * ((T.v[Y * TN + X] + T.v[Y * TN + X1]) + (T.v[Y1 * TN + X] + T.v[Y1 * TN + X1]));
+            v[y][0] += 0.25f * ((tv[Y * TN + X] + tv[Y * TN + X1]) + (tv[Y1 * TN + X] + tv[Y1 * TN + X1]));
         }
     }
     at_sweep<N, L, C, R>(t, f, v);
     at_sweep<N, L, C, R>(t, f, v);
 }
 
-// Diagonals of the one-warp levels from the threads' masks: the count over a 2^LEVELS square is
+// Diagonals of the first one-warp level from the threads' masks: the count over a 2^LEVELS square is
 // the lane's block of 2^LEVELS rows and the right lane's.
 template <int N>
 __device__ __forceinline__ void at_tail_diagonals(At<N> &t) {
     using K = AtCfg<N>;
     constexpr int TN = K::TN, LV = K::LEVELS, TR = K::RW >> LV;
     constexpr float area = 1.0f / (1 << (2 * LV));
-    const TailLvl<TN> T(t.sm + K::T);
-    const float tb2 = t.tb2 * area, d0 = t.tb1 + 4.0f * tb2;
+    float *td = t.sm + K::T + TN * TN;
+    const float d0 = t.tb1 + 4.0f * t.tb2 * area;
 #pragma unroll
     for (int Y = 0; Y < TR; ++Y) {
         const unsigned rows = t.mask & ((K::CW << LV) == 32 ? 0xffffffffu
                                                             : ((1u << ((K::CW << LV) & 31)) - 1u) << (Y * (K::CW << LV)));
         const int own = __popc(rows), both = own + __shfl_sync(0xffffffffu, own, t.right);
         if ((t.lane & 1) == 0 && t.lane < K::LU) {
-            const int i = (t.warp * TR + Y) * TN + (t.lane >> 1);
-            T.d[i] = fmaf((float)both, t.icg * area, d0);
-            T.w[i] = __fdividef(AS_OMEGA, T.d[i]);
-        }
-    }
-    if constexpr (K::TN2 > 0) {
-        __syncthreads();
-        if (t.warp == 0) {
-            constexpr int n2 = K::TN2;
-            const TailLvl<n2> B(t.sm + K::T2);
-            const float e0 = t.tb1 + tb2;  // 4 (tb2 / 4)
-            tail_for<n2>(t.lane, [&](int Y, int X, int i) {
-                const float *d = T.d + 2 * Y * TN + 2 * X;
-                const float m = 0.25f * ((d[0] + d[1]) + (d[TN] + d[TN + 1])) - d0;  // mean of m icg
-                B.d[i] = e0 + m;
-                B.w[i] = __fdividef(AS_OMEGA, B.d[i]);
-            });
+            td[(t.warp * TR + Y) * TN + (t.lane >> 1)] = fmaf((float)both, t.icg * area, d0);
         }
     }
 }
@@ -462,6 +492,10 @@ __global__ void __launch_bounds__(AtCfg<N>::NT, MINB) active_set_tile_kernel(con
     t.tb1 = (float)tb1;
     t.icg = (float)icg;
     t.tb2 = (float)tb2h;
+    t.d0 = t.tb1 + 4.0f * t.tb2;
+    t.d1 = t.d0 + t.icg;
+    t.w0 = AS_OMEGA / t.d0;
+    t.w1 = AS_OMEGA / t.d1;
     for (int i = threadIdx.x; i < nn; i += K::NT) U[i] = (double)a.u0[smp * (size_t)nn + i];
     __syncthreads();
     bool failed = false;
