@@ -12,6 +12,7 @@
 
 #include "mfmc_internal.h"
 #include "tma_step.cuh"
+#include "trace.cuh"
 
 namespace mfmc {
 
@@ -352,7 +353,8 @@ static mfmc_status solve_impl(mfmc_model *m, int algo, const double *eps, const 
                                       (uintptr_t)u0, (uintptr_t)uT, (uintptr_t)ubar, (uintptr_t)ooi,
                                       (uintptr_t)st, (uintptr_t)m->coef, (uintptr_t)m->bufA, (uintptr_t)m->bufB,
                                       (uintptr_t)m->padA, (uintptr_t)m->padB, (uintptr_t)m->partials,
-                                      (uintptr_t)m->map_sw, (uintptr_t)m->map_sh, (uintptr_t)m->d_wtab};
+                                      (uintptr_t)m->map_sw, (uintptr_t)m->map_sh, (uintptr_t)m->d_wtab,
+                                      (uintptr_t)trace_buf().rec};
     };
     if (graphable && m->gexec && m->gkey == key()) {
         MFMC_CUDA(cudaGraphLaunch(m->gexec, st));

@@ -1,5 +1,5 @@
-// Spectral step on this library's own FFT kernels (MFMC_ALGO_SPECTRAL): n = 1024 here, n = 64 and
-// 128 in the resident register-transform form below, other even n <= 128 in the resident
+// Spectral step on this library's own FFT kernels (MFMC_ALGO_SPECTRAL): n = 1024 here, n = 64, 88
+// and 128 in the resident tile form (spectral_tile.cuh), other even n <= 128 in the resident
 // mixed-radix form (spectral_resident.cu).
 //
 // On the periodic lattice the nodal quadrature (gamma * u)_i = sum_{z in D} w_z u_{i+z}
@@ -32,6 +32,7 @@
 
 #include "mfmc_internal.h"
 #include "spectral_queue.cuh"
+#include "spectral_tile.cuh"
 #include "tma_step.cuh"
 
 namespace mfmc {
@@ -348,231 +349,11 @@ timeout:
     }
 }
 
-// ----------------------------------------------------------------------------- small lattices
-// n = 32 E with E = 2 or 4 (n = 64, 128: the paper's meshes h = 1/64 and 1/128): a CTA keeps its
-// samples' fields and half spectra in shared memory for every step (one sample at n = 128, four
-// at n = 64) and writes only the final fields and their OoI.  A warp transforms 32 / E
-// sequences of length n at once, E lanes each: every lane transforms its 32 values (stride E)
-// in registers, multiplies by W_n^(n1 k2), and after an exchange through the warp's scratch
-// takes E-point DFTs across the E lanes (four-step with n = E x 32).
-template <int E>
-struct SmallCfg {
-    static constexpr int N = 32 * E, NH = N / 2 + 1;
-    static constexpr int F = 32 / E;                         // transforms per warp
-    static constexpr int Q = 32 / E;                         // k2 values per lane after the exchange
-    static constexpr int SPC = (128 / N) * (128 / N);        // samples per CTA
-    static constexpr int WARPS = 9;                          // 8 for the row pairs, 9 for the columns
-    // the field in rows of RS = N + 1 floats (the row pairs a warp transforms then start in
-    // different banks), then the half spectrum (N RS is even: 8-byte aligned)
-    static constexpr int RS = N + 1;
-    static constexpr int SAMPLE_FLOATS = N * RS + 2 * N * NH;
-    // a warp's scratch (complex values): the exchange of warp_fft_small (1024) and the forward
-    // row pass's staging of its F transforms, each padded by one value (F (N + 1) >= 1024)
-    static constexpr int SCR = F * (N + 1);
-    static constexpr size_t SMEM = ((size_t)SPC * SAMPLE_FLOATS + 2 * (WARPS * SCR + E * 33)) * sizeof(float);
-};
-
-// E lanes per transform (lane t: transform f = t / E, n1 = t % E).  On entry lane (f, n1) holds
-// x_f[n1 + E j] in v[j]; on return X_f[k2 + 32 k1] with k2 = n1 Q + q in v[q E + k1] (Q = 32 / E).
-// scr: the warp's 1024 complex values of scratch; tw: W_n^(n1 k2) at tw[n1 * 33 + k2].
-// The exchange stores element (f, k2, n1) in slot n1 ^ (k2 / Q) of its row of E, so that both
-// the stores (fixed k2) and the loads (k2 = n1 Q + q, fixed q and m) touch every bank once.
-template <int E, bool INV>
-__device__ __forceinline__ void warp_fft_small(float2 (&v)[kSq], float2 *scr, const float2 *tw, int t) {
-    constexpr int Q = 32 / E;
-    const int f = t / E, n1 = t - f * E;
-    fft32<INV>(v);  // Y_f[n1][k2] = sum_j x_f[n1 + E j] W_32^(j k2), in v[brev5(k2)]
-    // Y_f[n1][k2] W_n^(n1 k2) to scratch element (32 f + ((k2 + f) mod 32)) E + (n1 ^ (k2 / Q))
-#pragma unroll
-    for (int k2 = 0; k2 < kSq; ++k2)
-        scr[(f * kSq + ((k2 + f) & 31)) * E + (n1 ^ (k2 / Q))] = cmulw<INV>(v[brev5(k2)], tw[n1 * 33 + k2]);
-    __syncwarp();
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-        const int k2 = n1 * Q + q;
-        float2 y[E];
-#pragma unroll
-        for (int m = 0; m < E; ++m) y[m] = scr[(f * kSq + ((k2 + f) & 31)) * E + (m ^ n1)];  // k2 / Q = n1
-        if constexpr (E == 2) {
-            v[q * 2 + 0] = cadd(y[0], y[1]);
-            v[q * 2 + 1] = csub(y[0], y[1]);
-        } else {  // E = 4: W_4 = -i (inverse: +i)
-            const float2 s02 = cadd(y[0], y[2]), d02 = csub(y[0], y[2]);
-            const float2 s13 = cadd(y[1], y[3]), d13 = csub(y[1], y[3]);
-            const float2 r13 = INV ? make_float2(-d13.y, d13.x) : make_float2(d13.y, -d13.x);
-            v[q * 4 + 0] = cadd(s02, s13);
-            v[q * 4 + 2] = csub(s02, s13);
-            v[q * 4 + 1] = cadd(d02, r13);
-            v[q * 4 + 3] = csub(d02, r13);
-        }
-    }
-    __syncwarp();
-}
-
-// The whole solve of SPC samples per CTA on an n x n lattice, n = 32 E.  Per step: row pass
-// (pairs of rows packed as one complex row, forward transform, split into the two half spectra),
-// column pass (forward over y, product with khatT[kx][ky] = K^(ky, kx) / n^2, inverse), row pass
-// (the two half-spectrum rows of a pair combined, inverse transform: S on both rows, update and
-// projection in place).  Then the final fields to uT (when given) and the per-sample FP64 mean
-// in a fixed order.  The samples s0 .. s0 + nloc - 1 (nloc <= SPC) by the CTA's C::WARPS warps;
-// with STEPS, sample s takes steps_ps[s] steps (a sample whose steps are done keeps its field
-// while the others go on), else every sample nsteps.  sm_small: C::SMEM bytes of shared memory;
-// red: C::WARPS * 32 doubles.
-template <int E, bool STEPS>
-__device__ __forceinline__ void small_solve(const float *u0, float *uT, const StepCoef *coef, const float *khatT,
-                                            const float2 *twg, int s0, int nloc, const int *steps_ps, int nsteps,
-                                            double *ubar, double *ooi, float *sm_small, double *red) {
-    using C = SmallCfg<E>;
-    constexpr int N = C::N, NH = C::NH, F = C::F, Q = C::Q, SPC = C::SPC;
-    float2 *scr_all = reinterpret_cast<float2 *>(sm_small + SPC * C::SAMPLE_FLOATS);
-    float2 *tw = scr_all + C::WARPS * C::SCR;
-    const int w = threadIdx.x >> 5, t = threadIdx.x & 31, f = t / E, n1 = t - f * E;
-    float2 *scr = scr_all + w * C::SCR;
-    auto steps_of = [&](int s) { return s >= nloc ? 0 : steps_ps[s0 + s]; };
-    int kmax = nsteps;
-    if constexpr (STEPS) {
-        kmax = 0;
-        for (int s = 0; s < nloc; ++s) kmax = max(kmax, steps_of(s));
-    }
-    auto fld = [&](int s) { return sm_small + s * C::SAMPLE_FLOATS; };
-    auto spc = [&](int s) { return reinterpret_cast<float2 *>(sm_small + s * C::SAMPLE_FLOATS + N * C::RS); };
-    for (int i = threadIdx.x; i < SPC * N * N; i += blockDim.x) {
-        const int s = i / (N * N), r = i - s * N * N;
-        fld(s)[(r / N) * C::RS + r % N] = s < nloc ? u0[(size_t)(s0 + s) * N * N + r] : 0.f;
-    }
-    for (int i = threadIdx.x; i < E * 33; i += blockDim.x) tw[i] = twg[i];
-    __syncthreads();
-    for (int step = 0; step < kmax; ++step) {
-        if (w < 8) {  // forward row pass: pair p of the CTA's SPC * n / 2 pairs
-            const int p = w * F + f, s = p / (N / 2), y = 2 * (p - s * (N / 2));
-            const float *ua = fld(s) + y * C::RS, *ub = ua + C::RS;
-            float2 v[kSq];
-#pragma unroll
-            for (int j = 0; j < kSq; ++j) v[j] = make_float2(ua[n1 + E * j], ub[n1 + E * j]);
-            warp_fft_small<E, false>(v, scr, tw, t);
-#pragma unroll
-            for (int q = 0; q < Q; ++q)
-#pragma unroll
-                for (int k1 = 0; k1 < E; ++k1) scr[f * (N + 1) + n1 * Q + q + kSq * k1] = v[q * E + k1];
-            __syncwarp();
-            float2 *sa = spc(s) + y * NH, *sb = sa + NH;
-#pragma unroll
-            for (int i = 0; i <= N / 2 / E; ++i) {
-                const int k = n1 + E * i;
-                if (k <= N / 2) {
-                    const float2 zk = scr[f * (N + 1) + k], zm = scr[f * (N + 1) + ((N - k) & (N - 1))];
-                    sa[k] = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
-                    sb[k] = make_float2(0.5f * (zk.y + zm.y), 0.5f * (zm.x - zk.x));
-                }
-            }
-            __syncwarp();
-        }
-        __syncthreads();
-        {  // column pass: slot w + 9 f of the CTA's SPC * (n / 2 + 1) columns
-            const int slot = w + C::WARPS * f;
-            const bool active = slot < SPC * NH && slot / NH < nloc;
-            const int sl = active ? slot : 0, s = sl / NH, c = sl - s * NH;
-            float2 *col = spc(s) + c;  // element ky at col[ky * NH]
-            float2 v[kSq];
-#pragma unroll
-            for (int j = 0; j < kSq; ++j) v[j] = col[(n1 + E * j) * NH];
-            warp_fft_small<E, false>(v, scr, tw, t);
-            const float *kh = khatT + (size_t)c * N;
-#pragma unroll
-            for (int q = 0; q < Q; ++q)
-#pragma unroll
-                for (int k1 = 0; k1 < E; ++k1) {
-                    const int k = n1 * Q + q + kSq * k1;
-                    const float kk = __ldg(kh + k);
-                    if (active) col[k * NH] = make_float2(v[q * E + k1].x * kk, v[q * E + k1].y * kk);
-                }
-            __syncwarp();
-#pragma unroll
-            for (int j = 0; j < kSq; ++j) v[j] = col[(n1 + E * j) * NH];
-            warp_fft_small<E, true>(v, scr, tw, t);
-#pragma unroll
-            for (int q = 0; q < Q; ++q)
-#pragma unroll
-                for (int k1 = 0; k1 < E; ++k1)
-                    if (active) col[(n1 * Q + q + kSq * k1) * NH] = v[q * E + k1];
-        }
-        __syncthreads();
-        if (w < 8) {  // inverse row pass and the update
-            const int p = w * F + f, s = p / (N / 2), y = 2 * (p - s * (N / 2));
-            const float2 *sa = spc(s) + y * NH, *sb = sa + NH;
-            float2 v[kSq];
-#pragma unroll
-            for (int j = 0; j < kSq; ++j) {
-                const int k = n1 + E * j;
-                if (k <= N / 2) {
-                    const float2 a = sa[k], b = sb[k];
-                    v[j] = make_float2(a.x - b.y, a.y + b.x);
-                } else {
-                    const float2 a = sa[N - k], b = sb[N - k];
-                    v[j] = make_float2(a.x + b.y, b.x - a.y);
-                }
-            }
-            warp_fft_small<E, true>(v, scr, tw, t);  // S_y + i S_{y+1} at x = n1 Q + q + 32 k1
-            const StepCoef cf = coef[s0 + (s < nloc ? s : 0)];
-            float *ua = fld(s) + y * C::RS, *ub = ua + C::RS;
-            bool live = true;
-            if constexpr (STEPS) live = step < steps_of(s);  // else the sample's steps are done
-#pragma unroll
-            for (int q = 0; q < Q; ++q)
-#pragma unroll
-                for (int k1 = 0; k1 < E; ++k1) {
-                    const int x = n1 * Q + q + kSq * k1;
-                    const float2 S = v[q * E + k1];
-                    const float u0v = ua[x], u1v = ub[x];
-                    const float v0 = u0v + fmaf(cf.c1, fmaf(-cf.c0, u0v, S.x), cf.c2 * u0v);
-                    const float v1 = u1v + fmaf(cf.c1, fmaf(-cf.c0, u1v, S.y), cf.c2 * u1v);
-                    if (live) {
-                        ua[x] = fminf(1.f, fmaxf(-1.f, v0));
-                        ub[x] = fminf(1.f, fmaxf(-1.f, v1));
-                    }
-                }
-        }
-        __syncthreads();
-    }
-    for (int s = 0; s < nloc; ++s) {
-        const float *u = fld(s);
-        double acc = 0.0;
-        for (int i = threadIdx.x; i < N * N; i += blockDim.x) {
-            const float x = u[(i / N) * C::RS + i % N];
-            acc += (double)x;
-            if (uT) uT[(size_t)(s0 + s) * N * N + i] = x;
-        }
-        red[threadIdx.x] = acc;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double tot = 0.0;
-            for (int i = 0; i < C::WARPS * 32; ++i) tot += red[i];
-            const double mean = tot / ((double)N * N);
-            if (ubar) ubar[s0 + s] = mean;
-            if (ooi) ooi[s0 + s] = 0.5 * (1.0 + mean);
-        }
-        __syncthreads();
-    }
-}
-
-template <int E>
-__global__ void __launch_bounds__(SmallCfg<E>::WARPS * 32, 1)
-    spectral_small_kernel(const float *u0, float *uT, const StepCoef *coef, const float *khatT, const float2 *twg,
-                          int ns, int nsteps, double *ubar, double *ooi) {
-    using C = SmallCfg<E>;
-    extern __shared__ __align__(16) float sm_small[];
-    __shared__ double red[C::WARPS * 32];
-    const int s0 = blockIdx.x * C::SPC;
-    const int nloc = ns - s0 < C::SPC ? ns - s0 : C::SPC;
-    small_solve<E, false>(u0, uT, coef, khatT, twg, s0, nloc, nullptr, nsteps, ubar, ooi, sm_small, red);
-}
-
 // ----------------------------------------------------------------------------- the queue
 // One sample's whole solve on the mixed-radix transforms (any even n <= 128 they serve): the
 // field in shared memory, per step the disc sums of cta_disc_sums written straight into the
 // update and projection (the pair's rows are no longer read by the transforms then), at the end
-// the field to uT and the FP64 mean in a fixed order.  N > 0: n == N on the compile-time plan.
-template <int N>
+// the field to uT and the FP64 mean in a fixed order.
 __device__ __noinline__ void sq_solve_generic(const SqModelDev &M, int s, float *smem, double *red) {
     const int n = M.plan.n, nn = n * n;
     float *u = smem;
@@ -582,7 +363,7 @@ __device__ __noinline__ void sq_solve_generic(const SqModelDev &M, int s, float 
     const StepCoef cf = M.coef[s];
     const int steps = M.steps_ps ? M.steps_ps[s] : M.nsteps;
     for (int k = 0; k < steps; ++k)
-        cta_disc_sums<N, float>(
+        cta_disc_sums<0, float>(
             M.plan, fsm, M.khat, M.tw, [&](int y, int x) { return u[y * n + x]; },
             [&](int y, int x, float S) {
                 const float uv = u[y * n + x];
@@ -600,7 +381,7 @@ __device__ __noinline__ void sq_solve_generic(const SqModelDev &M, int s, float 
     __syncthreads();
     if (threadIdx.x == 0) {
         double tot = 0.0;
-        for (int i = 0; i < kSqThreads; ++i) tot += red[i];
+        for (int i = 0; i < (int)blockDim.x; ++i) tot += red[i];
         const double mean = tot / (double)nn;
         if (M.ubar) M.ubar[s] = mean;
         if (M.ooi) M.ooi[s] = 0.5 * (1.0 + mean);
@@ -608,48 +389,69 @@ __device__ __noinline__ void sq_solve_generic(const SqModelDev &M, int s, float 
     __syncthreads();  // the field and red are free for the next item
 }
 
+// Sample s of a tile-form model by the CTA's warps w0 .. w0 + N / 8 - 1.
+template <int N>
+__device__ __forceinline__ void sq_tile(const SqModelDev &M, int s, float2 *smem, double *red, int w0, int bar) {
+    constexpr size_t nn = (size_t)N * N;
+    tile_solve<N>(M.u0 + s * nn, M.uT ? M.uT + s * nn : nullptr, M.coef[s], M.tab, M.tw,
+                  M.steps_ps ? M.steps_ps[s] : M.nsteps, M.ubar ? M.ubar + s : nullptr, M.ooi ? M.ooi + s : nullptr,
+                  smem, red, (int)(threadIdx.x >> 5) - w0, bar);
+}
+
 // Persistent CTAs take (model, sample group) items through an atomic ticket counter, heaviest
 // model first (the host orders the models), and run each with the fastest form for its lattice.
-// SMALL: the launch has register-form items (n = 64, 128), whose 160-odd registers allow one CTA
-// per SM; without them the mixed-radix items alone fit two CTAs per SM.
-template <bool SMALL>
-__global__ void __launch_bounds__(kSqThreads, SMALL ? 1 : 2) spectral_queue_kernel(const __grid_constant__ SqArgs a) {
+// TILE: the launch has tile-form items (n = 64, 88, 128): sixteen warps, of which a 128^2 sample
+// takes all, an 88^2 sample eleven and each half two of a 64^2 item's four samples.  Without them
+// nine warps at fewer registers, two CTAs per SM.
+template <bool TILE>
+__global__ void __launch_bounds__(TILE ? kSqTileThreads : kSqThreads, TILE ? 1 : 2)
+    spectral_queue_kernel(const __grid_constant__ SqArgs a) {
     extern __shared__ __align__(16) float sq_smem[];
-    __shared__ double red[kSqThreads];
+    __shared__ double red[TILE ? kSqTileThreads : kSqThreads];
     __shared__ int item;
     for (;;) {
+        __syncthreads();  // the item before is done: its ticket and shared memory are free
         if (threadIdx.x == 0) item = atomicAdd(a.counter, 1);
         __syncthreads();
         const int it = item;
-        __syncthreads();  // every thread has read the ticket before thread 0 takes the next
         if (it >= a.total) break;
         const unsigned long long t0 = a.trace.rec ? trace_clock() : 0ull;
         int k = 0;
         while (k + 1 < a.nm && it >= a.begin[k + 1]) ++k;
         const SqModelDev &M = a.m[k];
         const int local = it - a.begin[k];
-        if (SMALL && M.kind == kSqSmall128) {
-            if (M.steps_ps)
-                small_solve<4, true>(M.u0, M.uT, M.coef, M.khat, M.tw, local, 1, M.steps_ps, M.nsteps, M.ubar, M.ooi,
-                                     sq_smem, red);
-            else
-                small_solve<4, false>(M.u0, M.uT, M.coef, M.khat, M.tw, local, 1, nullptr, M.nsteps, M.ubar, M.ooi,
-                                      sq_smem, red);
-        } else if (SMALL && M.kind == kSqSmall64) {
-            const int s0 = local * SmallCfg<2>::SPC, nloc = min(SmallCfg<2>::SPC, M.ns - s0);
-            if (M.steps_ps)
-                small_solve<2, true>(M.u0, M.uT, M.coef, M.khat, M.tw, s0, nloc, M.steps_ps, M.nsteps, M.ubar, M.ooi,
-                                     sq_smem, red);
-            else
-                small_solve<2, false>(M.u0, M.uT, M.coef, M.khat, M.tw, s0, nloc, nullptr, M.nsteps, M.ubar, M.ooi,
-                                      sq_smem, red);
-        } else if (M.plan.n == 88) {
-            sq_solve_generic<88>(M, local, sq_smem, red);
+        if constexpr (TILE) {
+            float2 *sm = reinterpret_cast<float2 *>(sq_smem);
+            const int w = threadIdx.x >> 5;
+            if (M.kind == kSqTile128) {
+                sq_tile<128>(M, local, sm, red, 0, 1);
+            } else if (M.kind == kSqTile64) {
+                const int g = w >> 3, s0 = local * 4, n = min(4, M.ns - s0);
+                float2 *gs = sm + g * (hf_smem_bytes<64, float>() / sizeof(float2));
+                for (int s = g; s < n; s += 2) sq_tile<64>(M, s0 + s, gs, red + 8 * g, 8 * g, 1 + g);
+            } else if (M.kind == kSqTile88) {
+                if (w < HfCfg<88>::NW) sq_tile<88>(M, local, sm, red, 0, 1);
+            } else {
+                sq_solve_generic(M, local, sq_smem, red);
+            }
+            __syncthreads();  // every warp's part is done
         } else {
-            sq_solve_generic<0>(M, local, sq_smem, red);
+            sq_solve_generic(M, local, sq_smem, red);
         }
         if (threadIdx.x == 0) trace_put(a.trace, kTraceSpectralQueue, (uint32_t)it, 0, t0);
     }
+}
+
+// One sample per CTA (a batch of one tile-form model).
+template <int N, int MINB>
+__global__ void __launch_bounds__(HfCfg<N>::NT, MINB) spectral_tile_kernel(const __grid_constant__ SqModelDev M, int s0,
+                                                                           TraceBuf trace) {
+    extern __shared__ __align__(16) float sq_smem[];
+    __shared__ double red[HfCfg<N>::NW];
+    const unsigned long long t0 = trace.rec ? trace_clock() : 0ull;
+    const int s = s0 + blockIdx.x;
+    sq_tile<N>(M, s, reinterpret_cast<float2 *>(sq_smem), red, 0, 0);
+    if (threadIdx.x == 0) trace_put(trace, kTraceSpectralQueue, (uint32_t)s, 0, t0);
 }
 
 // ----------------------------------------------------------------------------- host side
@@ -660,9 +462,8 @@ struct SpectralState {
     float2 *spec = nullptr;   // [cap][1024][528]
     float *bufA = nullptr, *bufB = nullptr;
     float2 *tw = nullptr;     // [32][32]: W_1024^(t k) at [k][t]
-    int small_n = 0;          // n = 64 or 128: the resident form's tables
-    float *khat_small = nullptr;   // [n/2 + 1][n]: K^(ky, kx) / n^2 at [kx][ky]
-    float2 *tw_small = nullptr;    // [E][33]: W_n^(n1 k2) at [n1][k2]
+    float4 *tab = nullptr;     // n = 64, 88, 128: the tile form's product table and twiddles
+    float2 *twt = nullptr;
 };
 
 void spectral_release(SpectralState *s) {
@@ -672,21 +473,21 @@ void spectral_release(SpectralState *s) {
     cudaFree(s->bufA);
     cudaFree(s->bufB);
     cudaFree(s->tw);
-    cudaFree(s->khat_small);
-    cudaFree(s->tw_small);
+    cudaFree(s->tab);
+    cudaFree(s->twt);
     delete s;
 }
 
 bool spectral_supported(const Model &m) {
     const int n = m.d.n;
-    return ((n == kN || n == 128 || n == 64) && m.d.bc == MFMC_BC_PERIODIC && m.d.beta2 == 0.0 && 2 * m.R + 1 <= n) ||
+    return ((n == kN || hf_supported(n)) && m.d.bc == MFMC_BC_PERIODIC && m.d.beta2 == 0.0 && 2 * m.R + 1 <= n) ||
            spectral_resident_supported(m);
 }
 
 // K^(ky, kx) = sum_dy cos(2 pi ky dy / n) sum_{dx: (dx, dy) in D} w cos(2 pi kx dx / n) (the
 // sine terms cancel: the disc and the weights are even in dx and in dy), in FP64 on the host,
 // with the weights the FP32 kernels use; divided by n^2 for the two unnormalised inverses.
-std::vector<float> spectral_khat(const Model &m, int n) {
+static std::vector<double> spectral_khat64(const Model &m, int n) {
     const int R = m.R, half = n / 2 + 1;
     std::vector<double> cs(n);
     for (int i = 0; i < n; ++i) cs[i] = std::cos(2.0 * M_PI * (double)i / (double)n);
@@ -703,15 +504,20 @@ std::vector<float> spectral_khat(const Model &m, int n) {
             A[(size_t)dy * half + kx] = s;
         }
     }
-    std::vector<float> kh((size_t)half * n);
+    std::vector<double> kh((size_t)half * n);
     const double scale = 1.0 / ((double)n * n);
     for (int ky = 0; ky < n; ++ky)
         for (int kx = 0; kx < half; ++kx) {
             double s = A[kx];  // dy = 0
             for (int dy = 1; dy <= R; ++dy) s += 2.0 * cs[(size_t)((long long)ky * dy % n)] * A[(size_t)dy * half + kx];
-            kh[(size_t)kx * n + ky] = (float)(s * scale);
+            kh[(size_t)kx * n + ky] = s * scale;
         }
     return kh;
+}
+
+std::vector<float> spectral_khat(const Model &m, int n) {
+    const std::vector<double> k = spectral_khat64(m, n);
+    return std::vector<float>(k.begin(), k.end());
 }
 
 // The register transforms' twiddles (c_w32), written once per device before the first
@@ -784,87 +590,77 @@ static mfmc_status spectral_prepare(Model &m, size_t ns) {
     return MFMC_OK;
 }
 
-// The register form's tables for n = 32 E (once per model and device): K^ / n^2 at [kx][ky] and
-// W_n^(n1 k2) at [n1][k2]; the register transforms' constants first.
-template <int E>
-static mfmc_status small_tables(Model &m, const float **khatT, const float2 **twp) {
-    using C = SmallCfg<E>;
-    constexpr int N = C::N;
+mfmc_status spectral_tile_tables(Model &m, const float4 **tab, const float2 **tw) {
+    const int n = m.d.n;
+    if (!hf_supported(n)) return fail(MFMC_EINVAL, "the tile form serves n = 64, 88 and 128");
     int dev = 0;
     MFMC_CUDA(cudaGetDevice(&dev));
-    {
-        const mfmc_status cs = spectral_constants();
-        if (cs != MFMC_OK) return cs;
-    }
     if (!m.spectral) m.spectral = new SpectralState();
     SpectralState &f = *m.spectral;
-    if (f.dev != dev || f.small_n != N || !f.khat_small) {
-        cudaFree(f.khat_small);
-        cudaFree(f.tw_small);
-        f.khat_small = nullptr;
-        f.tw_small = nullptr;
-        const std::vector<float> kh = spectral_khat(m, N);
-        std::vector<float2> tw((size_t)E * 33, make_float2(0.f, 0.f));
-        for (int n1 = 0; n1 < E; ++n1)
-            for (int k2 = 0; k2 < kSq; ++k2) {
-                const long long e = (long long)n1 * k2 % N;
-                tw[(size_t)n1 * 33 + k2] =
-                    make_float2((float)std::cos(2.0 * M_PI * e / N), (float)-std::sin(2.0 * M_PI * e / N));
-            }
-        MFMC_CUDA(cudaMalloc((void **)&f.khat_small, kh.size() * sizeof(float)));
-        MFMC_CUDA(cudaMemcpy(f.khat_small, kh.data(), kh.size() * sizeof(float), cudaMemcpyHostToDevice));
-        MFMC_CUDA(cudaMalloc((void **)&f.tw_small, tw.size() * sizeof(float2)));
-        MFMC_CUDA(cudaMemcpy(f.tw_small, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice));
-        f.small_n = N;
+    if (f.dev != dev || !f.tab || !f.twt) {
+        cudaFree(f.tab);
+        cudaFree(f.twt);
+        f.tab = nullptr;
+        f.twt = nullptr;
+        const std::vector<double> kh = spectral_khat64(m, n);  // [kx][ky]
+        std::vector<float> tb((size_t)4 * (n / 2 + 1) * (n / 2)), t2((size_t)2 * hf_tw_size(n));
+        hf_product_table<float>(n, [&](int kx, int ky) { return kh[(size_t)kx * n + ky]; }, tb.data());
+        hf_twiddles<float>(n, t2.data());
+        MFMC_CUDA(cudaMalloc((void **)&f.tab, tb.size() * sizeof(float)));
+        MFMC_CUDA(cudaMemcpy(f.tab, tb.data(), tb.size() * sizeof(float), cudaMemcpyHostToDevice));
+        MFMC_CUDA(cudaMalloc((void **)&f.twt, t2.size() * sizeof(float)));
+        MFMC_CUDA(cudaMemcpy(f.twt, t2.data(), t2.size() * sizeof(float), cudaMemcpyHostToDevice));
         f.dev = dev;
     }
-    *khatT = f.khat_small;
-    *twp = f.tw_small;
+    *tab = f.tab;
+    *tw = f.twt;
     return MFMC_OK;
 }
 
-mfmc_status spectral_small_tables(Model &m, const float **khatT, const float2 **tw) {
-    if (m.d.n == 128) return small_tables<4>(m, khatT, tw);
-    if (m.d.n == 64) return small_tables<2>(m, khatT, tw);
-    return fail(MFMC_EINVAL, "the register-transform form serves n = 64 and 128");
+size_t spectral_queue_smem(int kind, int n, int warps) {
+    if (kind == kSqTile128) return hf_smem_bytes<128, float>();
+    if (kind == kSqTile88) return hf_smem_bytes<88, float>();
+    if (kind == kSqTile64) return 2 * hf_smem_bytes<64, float>();
+    return (size_t)n * n * sizeof(float) + fft_smem_bytes<float>(n, warps);
 }
 
-size_t spectral_queue_smem(int kind, int n) {
-    if (kind == kSqSmall128) return SmallCfg<4>::SMEM;
-    if (kind == kSqSmall64) return SmallCfg<2>::SMEM;
-    return (size_t)n * n * sizeof(float) + fft_smem_bytes<float>(n, kSqThreads / 32);
-}
-
-int spectral_queue_blocks_per_sm(bool small, size_t smem) {
-    auto kern = small ? spectral_queue_kernel<true> : spectral_queue_kernel<false>;
+int spectral_queue_blocks_per_sm(bool tile, size_t smem) {
+    auto kern = tile ? spectral_queue_kernel<true> : spectral_queue_kernel<false>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int per = 0;
-    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, kSqThreads, smem);
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, tile ? kSqTileThreads : kSqThreads, smem);
     (void)cudaGetLastError();  // a failed query must not be reported by a later launch check
     return e == cudaSuccess && per > 0 ? per : 1;
 }
 
-mfmc_status launch_spectral_queue(bool small, const SqArgs &a, int grid, size_t smem, cudaStream_t st) {
-    auto kern = small ? spectral_queue_kernel<true> : spectral_queue_kernel<false>;
+mfmc_status launch_spectral_queue(bool tile, const SqArgs &a, int grid, size_t smem, cudaStream_t st) {
+    auto kern = tile ? spectral_queue_kernel<true> : spectral_queue_kernel<false>;
     MFMC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    kern<<<grid, kSqThreads, smem, st>>>(a);
+    kern<<<grid, tile ? kSqTileThreads : kSqThreads, smem, st>>>(a);
     MFMC_LAUNCHED("spectral queue launch");
     return MFMC_OK;
 }
 
-// The resident form for n = 64 and 128: tables once per model, one launch for the whole solve.
-template <int E>
-static mfmc_status run_solve_spectral_small(Model &m, const StepCoef *coef, const float *u0, size_t ns, int nsteps,
-                                            float *uT, double *ubar, double *ooi, cudaStream_t st) {
-    using C = SmallCfg<E>;
-    const float *khatT = nullptr;
-    const float2 *tw = nullptr;
-    const mfmc_status s = small_tables<E>(m, &khatT, &tw);
+// The tile form on one model: tables once per model, one launch for the whole solve, one sample per
+// CTA (n = 64 four CTAs per SM, n = 88 two).
+template <int N, int MINB>
+static mfmc_status run_solve_spectral_tile(Model &m, const StepCoef *coef, const float *u0, size_t ns, int nsteps,
+                                           float *uT, double *ubar, double *ooi, cudaStream_t st) {
+    SqModelDev d{};
+    const mfmc_status s = spectral_tile_tables(m, &d.tab, &d.tw);
     if (s != MFMC_OK) return s;
-    auto kern = spectral_small_kernel<E>;
-    MFMC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM));
-    const unsigned grid = (unsigned)((ns + C::SPC - 1) / C::SPC);
-    kern<<<grid, C::WARPS * 32, C::SMEM, st>>>(u0, uT, coef, khatT, tw, (int)ns, nsteps, ubar, ooi);
+    d.u0 = u0;
+    d.uT = uT;
+    d.ubar = ubar;
+    d.ooi = ooi;
+    d.coef = coef;
+    d.nsteps = nsteps;
+    d.ns = (int)ns;
+    auto kern = spectral_tile_kernel<N, MINB>;
+    constexpr size_t smem = hf_smem_bytes<N, float>();
+    MFMC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // (a trace record per sample on n = 88 only, as the trace's description says)
+    kern<<<(unsigned)ns, HfCfg<N>::NT, smem, st>>>(d, 0, N == 88 ? trace_buf() : TraceBuf{});
     MFMC_LAUNCHED("spectral launch 4");
     return MFMC_OK;
 }
@@ -879,8 +675,9 @@ mfmc_status run_solve_spectral(Model &m, const StepCoef *coef, const float *u0, 
         MFMC_CUDA(cudaDeviceGetAttribute(&one, cudaDevAttrMaxGridDimX, 0));
         if (ns > (size_t)one) return fail(MFMC_EINVAL, "batch too large for the spectral path");
     }
-    if (m.d.n == 128) return run_solve_spectral_small<4>(m, coef, u0, ns, nsteps, uT, ubar, ooi, st);
-    if (m.d.n == 64) return run_solve_spectral_small<2>(m, coef, u0, ns, nsteps, uT, ubar, ooi, st);
+    if (m.d.n == 128) return run_solve_spectral_tile<128, 1>(m, coef, u0, ns, nsteps, uT, ubar, ooi, st);
+    if (m.d.n == 88) return run_solve_spectral_tile<88, 2>(m, coef, u0, ns, nsteps, uT, ubar, ooi, st);
+    if (m.d.n == 64) return run_solve_spectral_tile<64, 4>(m, coef, u0, ns, nsteps, uT, ubar, ooi, st);
     if (m.d.n != kN) return run_solve_spectral_resident(m, coef, u0, ns, nsteps, uT, ubar, ooi, st);
     mfmc_status s = spectral_prepare(m, ns);
     if (s != MFMC_OK) return s;

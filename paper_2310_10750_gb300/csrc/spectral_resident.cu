@@ -1,13 +1,12 @@
 // Host side of the resident spectral queue (spectral_queue.cuh): one launch over the samples of up
 // to kSrMaxModels periodic beta2 = 0 models on small lattices (n <= 128), for one model
-// (MFMC_ALGO_SPECTRAL on an n other than 64, 128 and 1024) or a hierarchy (the mixed batch).
+// (MFMC_ALGO_SPECTRAL on an n other than 64, 88, 128 and 1024) or a hierarchy (the mixed batch).
 //
 // The work is a queue of (model, sample group) items, heaviest model first.  Persistent CTAs take
 // items with an atomic ticket counter; an item is a whole solve kept in shared memory for every
-// step: on n = 128 (one sample) and n = 64 (four samples) by the register-transform form, on any
-// other even n whose odd part is a product of 3, 5, 7 and 11 by the mixed-radix transforms of
-// smem_fft.cuh (the paper's n = 88 on its compile-time plan), each step's disc sums going straight
-// into the update of Eq. (nonl_CH_nm) with beta2 = 0 and the projection of Eq.
+// step: on n = 128, 88 (one sample) and n = 64 (four samples) by the tile form, on any other even n
+// whose odd part is a product of 3, 5, 7 and 11 by the mixed-radix transforms of smem_fft.cuh, each
+// step's disc sums going straight into the update of Eq. (nonl_CH_nm) with beta2 = 0 and the projection of Eq.
 // (potential_obstacle).  So the samples of every fidelity of the paper's hierarchy (Section 4:
 // h in {1/128, 1/88, 1/64}, any horizon, the Gaussian kernel, delta/h = 16.5 included) run
 // together in one launch, and the cheap items of the coarse models fill the SMs while the fine
@@ -19,6 +18,7 @@
 #include <vector>
 
 #include "mfmc_internal.h"
+#include "half_fft.cuh"
 #include "spectral_queue.cuh"
 
 namespace mfmc {
@@ -60,7 +60,9 @@ mfmc_status run_spectral_queue(Model *const *models, const SrBatch *batches, int
     SqArgs a{};
     size_t smem = 0;
     long long total = 0;
-    bool small = false;
+    bool tile = false;  // any tile-form item: it sets the CTA's warps
+    for (int k = 0; k < nm; ++k) tile = tile || hf_supported(models[k]->d.n);
+    const int warps = (tile ? kSqTileThreads : kSqThreads) / 32;
     for (int k = 0; k < nm; ++k) {
         Model &m = *models[k];
         if (!spectral_resident_supported(m))
@@ -69,16 +71,15 @@ mfmc_status run_spectral_queue(Model *const *models, const SrBatch *batches, int
         const SrBatch &b = batches[k];
         SqModelDev &d = a.m[k];
         const int n = m.d.n;
-        d.kind = n == 128 ? kSqSmall128 : (n == 64 ? kSqSmall64 : kSqGeneric);
-        d.spc = d.kind == kSqSmall64 ? 4 : 1;
-        small = small || d.kind != kSqGeneric;
+        d.kind = n == 128 ? kSqTile128 : (n == 88 ? kSqTile88 : (n == 64 ? kSqTile64 : kSqGeneric));
+        d.spc = d.kind == kSqTile64 ? 4 : 1;
         if (d.kind == kSqGeneric) {
             mfmc_status s = sr_tables(m);
             if (s != MFMC_OK) return s;
             d.khat = m.d_khat32;
             d.tw = m.d_tw32;
         } else {
-            mfmc_status s = spectral_small_tables(m, &d.khat, &d.tw);
+            mfmc_status s = spectral_tile_tables(m, &d.tab, &d.tw);
             if (s != MFMC_OK) return s;
         }
         d.u0 = b.u0;
@@ -94,7 +95,7 @@ mfmc_status run_spectral_queue(Model *const *models, const SrBatch *batches, int
         total += (long long)((b.ns + d.spc - 1) / d.spc);
         if (b.ns > (size_t)INT32_MAX / 2 || total > INT32_MAX / 2)
             return fail(MFMC_EINVAL, "batch too large for the resident spectral form");
-        smem = std::max(smem, spectral_queue_smem(d.kind, n));
+        smem = std::max(smem, spectral_queue_smem(d.kind, n, warps));
     }
     a.begin[nm] = (int)total;
     a.nm = nm;
@@ -106,9 +107,9 @@ mfmc_status run_spectral_queue(Model *const *models, const SrBatch *batches, int
     MFMC_CUDA(cudaMemsetAsync(counter, 0, sizeof(int), st));
     a.counter = counter;
     a.trace = trace_buf();
-    const int per = spectral_queue_blocks_per_sm(small, smem);
+    const int per = spectral_queue_blocks_per_sm(tile, smem);
     const int grid = (int)std::min<long long>(total, (long long)sms * per);
-    return launch_spectral_queue(small, a, grid, smem, st);
+    return launch_spectral_queue(tile, a, grid, smem, st);
 }
 
 mfmc_status run_solve_spectral_resident(Model &m, const StepCoef *coef, const float *u0, size_t ns, int nsteps,
