@@ -42,6 +42,7 @@
 #include <vector>
 
 #include "active_set_tile.cuh"
+#include "half_fft.cuh"
 
 namespace mfmc {
 
@@ -539,7 +540,19 @@ mfmc_status run_solve_active_set(Model &m, const double *eps_dev, const float *u
     a.tw = nullptr;
     a.warm = 0;
     a.trace = trace_buf();
-    if (own) {
+    if (own && tile) {
+        const int n = m.d.n, nh = n / 2 + 1;
+        if (!m.d_khat64) {
+            const std::vector<double> K = khat64_host(m, n);  // [ky][kx]
+            std::vector<double> tab((size_t)4 * nh * (n / 2)), tw((size_t)2 * hf_tw_size(n));
+            hf_product_table<double>(n, [&](int kx, int ky) { return K[(size_t)ky * nh + kx]; }, tab.data());
+            hf_twiddles<double>(n, tw.data());
+            MFMC_CUDA(cudaMalloc((void **)&m.d_tw64, tw.size() * sizeof(double)));
+            MFMC_CUDA(cudaMemcpy(m.d_tw64, tw.data(), tw.size() * sizeof(double), cudaMemcpyHostToDevice));
+            MFMC_CUDA(cudaMalloc((void **)&m.d_khat64, tab.size() * sizeof(double)));
+            MFMC_CUDA(cudaMemcpy(m.d_khat64, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice));
+        }
+    } else if (own) {
         const int n = m.d.n;
         if (!m.d_khat64) {
             const std::vector<double> K = khat64_host(m, n);
@@ -572,10 +585,8 @@ mfmc_status run_solve_active_set(Model &m, const double *eps_dev, const float *u
         t.nsteps = nsteps;
         t.newton_max = a.newton_max;
         t.cg_max = a.cg_max;
-        t.own_fft = a.own_fft;
-        t.plan = a.plan;
-        t.khat = a.khat;
-        t.tw = a.tw;
+        t.tab = own ? reinterpret_cast<const AsFactor *>(m.d_khat64) : nullptr;
+        t.tw = own ? m.d_tw64 : nullptr;
         t.trace = a.trace;
         t.ahat = a.ahat;
         t.chat = a.chat;

@@ -24,6 +24,7 @@
 #include <algorithm>
 
 #include "active_set_tile.cuh"
+#include "spectral_tile.cuh"
 
 namespace mfmc {
 
@@ -458,6 +459,38 @@ __device__ __forceinline__ void at_tail_diagonals(At<N> &t) {
     }
 }
 
+// g = e2a (disc sums of u) + c_F u by the CTA: the transforms of half_fft.cuh in FP64.  smem:
+// hf_smem_bytes<N, double>() bytes.  Begins and ends with a CTA barrier.
+template <int N>
+__device__ __noinline__ void at_disc_sums(const double *U, double *G, const AsFactor *tab, const double2 *twg,
+                                          double2 *smem, double e2a, double cF) {
+    using K = HfCfg<N>;
+    Hf<N, double2> h;
+    double2 *tw = smem + K::Z;
+    h.z = smem;
+    h.tw = tw;
+    h.warp = threadIdx.x >> 5;
+    h.lane = threadIdx.x & 31;
+    __syncthreads();
+    for (int i = threadIdx.x; i < K::TW; i += K::NT) tw[i] = twg[i];
+    __syncthreads();
+    const size_t r0 = (size_t)(2 * h.my_row()) * N + h.n1();
+    double2 v[K::A];
+#pragma unroll
+    for (int j = 0; j < K::A; ++j) v[j] = make_double2(U[r0 + 8 * j], U[r0 + N + 8 * j]);
+    h.rows_forward(v);
+    __syncthreads();
+    h.columns(tab);
+    __syncthreads();
+    h.rows_inverse(v);
+#pragma unroll
+    for (int j = 0; j < K::A; ++j) {
+        G[r0 + 8 * j] = fma(e2a, v[j].x, cF * U[r0 + 8 * j]);
+        G[r0 + N + 8 * j] = fma(e2a, v[j].y, cF * U[r0 + N + 8 * j]);
+    }
+    __syncthreads();
+}
+
 template <int N, int MINB>
 __global__ void __launch_bounds__(AtCfg<N>::NT, MINB) active_set_tile_kernel(const __grid_constant__ AsTileArgs a) {
     using K = AtCfg<N>;
@@ -502,10 +535,8 @@ __global__ void __launch_bounds__(AtCfg<N>::NT, MINB) active_set_tile_kernel(con
     unsigned long long n_newton = 0, n_cg = 0;
     for (int step = 1; step <= a.nsteps && !failed; ++step) {
         // explicit part g = gamma * u + c_F u
-        if (a.own_fft) {
-            cta_disc_sums<N, double>(
-                a.plan, at_smem, a.khat, a.tw, [&](int y, int x) { return U[y * N + x]; },
-                [&](int y, int x, double S) { G[y * N + x] = e2a * S + a.cF * U[y * N + x]; });
+        if (a.tab) {
+            at_disc_sums<N>(U, G, a.tab, a.tw, reinterpret_cast<double2 *>(at_smem), e2a, a.cF);
         } else {
             for (int i = threadIdx.x; i < nn; i += K::NT) {
                 const int y = i / N, x = i - y * N;
@@ -715,7 +746,7 @@ template <int N, int MINB>
 mfmc_status at_launch(const AsTileArgs &a, unsigned grid, cudaStream_t st) {
     using K = AtCfg<N>;
     size_t smem = K::SMEM;
-    if (a.own_fft) smem = std::max(smem, fft_smem_bytes<double>(N, K::NW));
+    if (a.tab) smem = std::max(smem, hf_smem_bytes<N, double>());
     auto kern = active_set_tile_kernel<N, MINB>;
     MFMC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     kern<<<grid, K::NT, smem, st>>>(a);

@@ -4,7 +4,6 @@
 #pragma once
 
 #include "mfmc_internal.h"
-#include "smem_fft.cuh"
 #include "trace.cuh"
 
 namespace mfmc {
@@ -14,6 +13,10 @@ constexpr float AS_CG_RTOL = 1e-5f;   // max |J d + F| / max |F| that ends a cor
 constexpr int AS_NU = 2;              // damped-Jacobi sweeps before and after each coarse correction
 constexpr int AS_NU_COARSE = 16;
 constexpr float AS_OMEGA = 0.8f;
+
+struct alignas(16) AsFactor {
+    double x, y, z, w;  // a row of hf_product_table
+};
 
 struct AsTileArgs {
     const float *u0;
@@ -28,10 +31,9 @@ struct AsTileArgs {
     int widths[kMaxR + 1];
     int R, nsteps;
     int newton_max, cg_max;
-    int own_fft;         // the disc sums by cta_disc_sums (khat, tw) instead of the direct sum
-    FftPlan plan;
-    const double *khat;  // K^(ky, kx) / n^2 at [ky][n/2 + 1], FP64
-    const double2 *tw;   // W_n^j, j < n
+    // the disc sums by FFT: product table and twiddles of half_fft.cuh; nullptr: the direct sum
+    const AsFactor *tab;
+    const double2 *tw;
     TraceBuf trace;
     size_t s0;
     double ahat, chat, tau, beta1, beta2, cF;

@@ -102,8 +102,9 @@ struct Model {
     float2 *d_tw32 = nullptr;     // and W_n^j, j < n
     int sr_dev = -1;              // device of those tables
     int *sr_counter = nullptr;    // its ticket counter
-    double *d_khat64 = nullptr;   // beta2 > 0, own FFT: K^ / n^2 at [ky][n/2 + 1] (FP64)
-    double2 *d_tw64 = nullptr;    // and W_n^j, j < n
+    double *d_khat64 = nullptr;   // beta2 > 0, own FFT (FP64): K^ / n^2 at [ky][n/2 + 1], or on n = 64,
+                                  // 88, 128 the product table of half_fft.cuh
+    double2 *d_tw64 = nullptr;    // and W_n^j, j < n, or half_fft.cuh's twiddles
     unsigned long long *d_as_iters = nullptr;  // Newton and CG iterations of the last beta2 > 0 solve
     int as_newton_max = kAsNewtonMax;           // iteration bounds of the beta2 > 0 solver
     int as_cg_max = kAsCgMax;
