@@ -1,14 +1,16 @@
-// Resident (whole field in shared memory) kernels for R in {1, ..., 6, 8}.
+// Resident kernels (the whole solve of a sample on chip): the strip form for R <= 4, the
+// shared-memory form for R = 5, 6, 8.
+#include "resident_strip.cuh"
 #include "rows_step.cuh"
 
 namespace mfmc {
 
 ResidentFn resident_launcher(int R) {
     switch (R) {
-        case 1: return &launch_resident<1>;
-        case 2: return &launch_resident<2>;
-        case 3: return &launch_resident<3>;
-        case 4: return &launch_resident<4>;
+        case 1: return &launch_resident_strip<1>;
+        case 2: return &launch_resident_strip<2>;
+        case 3: return &launch_resident_strip<3>;
+        case 4: return &launch_resident_strip<4>;
         case 5: return &launch_resident<5>;
         case 6: return &launch_resident<6>;
         case 8: return &launch_resident<8>;

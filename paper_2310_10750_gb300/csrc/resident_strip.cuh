@@ -1,0 +1,239 @@
+// The resident solve for R <= 4: one CTA per sample, the field in registers for every step.
+//
+// A group of n / 4 lanes owns a strip of 4 NB whole rows (a lane four columns), so a row's window
+// comes from two neighbour lanes by shuffles and the periodic wrap is a lane index.  Every row's
+// segment sums are formed once per step, by its owner, and added to the 2R + 1 output rows they
+// belong to; sums for rows of the strips above and below go there as partial sums through shared
+// memory (two buffers in turn, one CTA barrier per step).  Results do not depend on NB: an output
+// row's sum is (its own block of four rows + the block above) + the block below, each block's rows
+// in ascending order, whether the blocks lie in one thread or in two.
+//
+// What bounds it: the FMA pipe (R = 4: 5.5 adds per point for the segment sums, 8 for the disc
+// rows, 4 for the update: 2.2K cycles of a 128^2 step on an SM) and the shuffles and exchanges
+// (2.0K cycles).  The kernel it replaces formed one segment difference per (row, output row) and
+// walked (16 + 2R) / 16 of the rows, at 7 warps an SM (195 registers).
+//
+// NB = 2 for throughput.  NB = 1 halves a step's serial chain at twice the exchange traffic: taken
+// when the batch leaves most of the chip idle (launch_resident_strip).
+#pragma once
+
+#include "step_kernels.cuh"
+
+namespace mfmc {
+
+// The segment sums of a block of four rows u (four columns a lane), added to the output rows of
+// the block (own), the R rows above it (up[k]: row k - R) and the R rows below (dn[k]: row 4 + k).
+template <int R>
+__device__ __forceinline__ void strip_block(const float (&u)[4][4], int left, int right, float2 (&up)[R][2],
+                                            float2 (&own)[4][2], float2 (&dn)[R][2]) {
+    constexpr DiscClasses<R> cls{};
+    constexpr int M = 2 + R;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        float v[4 + 2 * R], p[5 + 2 * R];
+#pragma unroll
+        for (int k = 0; k < R; ++k) {
+            v[k] = __shfl_sync(0xffffffffu, u[r][4 - R + k], left);
+            v[4 + R + k] = __shfl_sync(0xffffffffu, u[r][k], right);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[R + k] = u[r][k];
+        // centre sums: p[k] = sum of v[M .. k - 1] for k > M, of v[k .. M - 1] for k < M
+        p[M] = 0.f;
+        p[M + 1] = v[M];
+        p[M - 1] = v[M - 1];
+#pragma unroll
+        for (int q = 1; q < M; ++q) {
+            p[M + 1 + q] = p[M + q] + v[M + q];
+            p[M - 1 - q] = p[M - q] + v[M - 1 - q];
+        }
+#pragma unroll
+        for (int c = 0; c < cls.count; ++c) {
+            const int hw = cls.width[c];
+            float h[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int b = i + R - hw, e = i + R + hw + 1;
+                h[i] = hw == 0 ? v[R + i] : (b >= M ? p[e] - p[b] : (e <= M ? p[b] - p[e] : p[e] + p[b]));
+            }
+            const float2 h01 = make_float2(h[0], h[1]), h23 = make_float2(h[2], h[3]);
+            auto add = [&](float2 (&s)[2], bool first) {
+                s[0] = first ? h01 : __fadd2_rn(s[0], h01);
+                s[1] = first ? h23 : __fadd2_rn(s[1], h23);
+            };
+#pragma unroll
+            for (int y = -R; y < 4 + R; ++y) {
+                const int ady = r > y ? r - y : y - r;
+                if (ady <= R && cls.of[ady <= R ? ady : 0] == c) {
+                    const bool first = r == (y > R ? y - R : 0);  // the output row's first row in this block
+                    if (y < 0)
+                        add(up[y < 0 ? y + R : 0], first);
+                    else if (y < 4)
+                        add(own[y >= 0 && y < 4 ? y : 0], first);
+                    else
+                        add(dn[y >= 4 ? y - 4 : 0], first);
+                }
+            }
+        }
+    }
+}
+
+__host__ __device__ constexpr int strip_groups(int n) { return 32 / (n / 4); }          // strips per warp
+__host__ __device__ constexpr int strip_warps(int n, int nb) {
+    return (n / (4 * nb) + strip_groups(n) - 1) / strip_groups(n);
+}
+inline size_t strip_smem(int n, int R, int nb) {
+    const size_t ex = (size_t)2 * (n / (4 * nb)) * 2 * R * n * sizeof(float), red = (size_t)(n / 4) * (n / 4) * sizeof(double);
+    return ex > red ? ex : red;
+}
+
+template <int R, int NB>
+__global__ void __launch_bounds__(512) resident_strip_kernel(ResidentArgs a) {
+    static_assert(R <= 4, "a block's sums reach the adjacent blocks only");
+    extern __shared__ float4 smem4[];
+    const int n = a.n, L = n / 4, strips = n / (4 * NB), groups = strip_groups(n);
+    const int lane = threadIdx.x & 31, g = lane / L, cg = lane - g * L;
+    const int strip_w = (threadIdx.x >> 5) * groups + g;
+    const bool act = g < groups && strip_w < strips;
+    const int strip = act ? strip_w : 0;   // idle lanes follow strip 0 and store nothing
+    const int base = lane - cg, lanes = g < groups ? L : 32 - groups * L;
+    const int left = base + (cg == 0 ? lanes - 1 : cg - 1), right = base + (cg == lanes - 1 ? 0 : cg + 1);
+    const int cc = act ? cg : 0;
+    // exchange rows [buffer][strip][0: for the strip above, 1: for the strip below][R][L]
+    const int ex_strip = 2 * R * L, ex_buf = strips * ex_strip;
+    float4 *const mine = smem4 + strip * ex_strip + cc;
+    const float4 *const from_up = smem4 + (strip == 0 ? strips - 1 : strip - 1) * ex_strip + R * L + cc;
+    const float4 *const from_dn = smem4 + (strip == strips - 1 ? 0 : strip + 1) * ex_strip + cc;
+    const size_t nn = (size_t)n * n, off = (size_t)strip * 4 * NB * n + 4 * cc;
+    for (int sample = blockIdx.x; sample < a.ns; sample += gridDim.x) {
+        const float *__restrict__ src = a.u0 + (size_t)sample * nn + off;
+        float u[NB][4][4];
+#pragma unroll
+        for (int b = 0; b < NB; ++b)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const float4 t = __ldg(reinterpret_cast<const float4 *>(src + (size_t)(4 * b + r) * n));
+                u[b][r][0] = t.x, u[b][r][1] = t.y, u[b][r][2] = t.z, u[b][r][3] = t.w;
+            }
+        const StepCoef cf = a.coef[sample];
+        const float2 nc0 = make_float2(-cf.c0, -cf.c0), c1 = make_float2(cf.c1, cf.c1), c2 = make_float2(cf.c2, cf.c2);
+        const int nsteps = a.steps_ps ? a.steps_ps[sample] : a.nsteps;
+#pragma unroll 1
+        for (int step = 0; step < nsteps; ++step) {
+            const int buf = (step & 1) * ex_buf;
+            float2 up[NB][R][2], own[NB][4][2], dn[NB][R][2];
+#pragma unroll
+            for (int b = 0; b < NB; ++b) {
+                strip_block<R>(u[b], left, right, up[b], own[b], dn[b]);
+                if (act && b == 0) {
+#pragma unroll
+                    for (int k = 0; k < R; ++k)
+                        mine[buf + k * L] = make_float4(up[0][k][0].x, up[0][k][0].y, up[0][k][1].x, up[0][k][1].y);
+                }
+                if (act && b == NB - 1) {
+#pragma unroll
+                    for (int k = 0; k < R; ++k)
+                        mine[buf + (R + k) * L] = make_float4(dn[b][k][0].x, dn[b][k][0].y, dn[b][k][1].x, dn[b][k][1].y);
+                }
+            }
+            __syncthreads();
+#pragma unroll
+            for (int b = 0; b < NB; ++b)
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    float2 s0 = own[b][r][0], s1 = own[b][r][1];
+                    if (r < R) {  // from the block above
+                        float2 t0, t1;
+                        if (b == 0) {
+                            const float4 t = from_up[buf + r * L];
+                            t0 = make_float2(t.x, t.y);
+                            t1 = make_float2(t.z, t.w);
+                        } else {
+                            t0 = dn[b - 1 >= 0 ? b - 1 : 0][r < R ? r : 0][0];
+                            t1 = dn[b - 1 >= 0 ? b - 1 : 0][r < R ? r : 0][1];
+                        }
+                        s0 = __fadd2_rn(s0, t0);
+                        s1 = __fadd2_rn(s1, t1);
+                    }
+                    if (r >= 4 - R) {  // from the block below
+                        float2 t0, t1;
+                        const int k = r - (4 - R) >= 0 ? r - (4 - R) : 0;
+                        if (b == NB - 1) {
+                            const float4 t = from_dn[buf + k * L];
+                            t0 = make_float2(t.x, t.y);
+                            t1 = make_float2(t.z, t.w);
+                        } else {
+                            t0 = up[b + 1 < NB ? b + 1 : 0][k][0];
+                            t1 = up[b + 1 < NB ? b + 1 : 0][k][1];
+                        }
+                        s0 = __fadd2_rn(s0, t0);
+                        s1 = __fadd2_rn(s1, t1);
+                    }
+                    const float2 x0 = make_float2(u[b][r][0], u[b][r][1]), x1 = make_float2(u[b][r][2], u[b][r][3]);
+                    const float2 v0 = __fadd2_rn(x0, __ffma2_rn(c1, __ffma2_rn(nc0, x0, s0), __fmul2_rn(c2, x0)));
+                    const float2 v1 = __fadd2_rn(x1, __ffma2_rn(c1, __ffma2_rn(nc0, x1, s1), __fmul2_rn(c2, x1)));
+                    u[b][r][0] = fminf(1.f, fmaxf(-1.f, v0.x));
+                    u[b][r][1] = fminf(1.f, fmaxf(-1.f, v0.y));
+                    u[b][r][2] = fminf(1.f, fmaxf(-1.f, v1.x));
+                    u[b][r][3] = fminf(1.f, fmaxf(-1.f, v1.y));
+                }
+        }
+        // OoI: FP64 sums of the blocks of 4 x 4 values, then in block order per column group, then
+        // over the groups
+        __syncthreads();  // the last step's exchange rows have been read
+        double *red = reinterpret_cast<double *>(smem4);
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            double part = 0.0;
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                part += ((double)u[b][r][0] + (double)u[b][r][1]) + ((double)u[b][r][2] + (double)u[b][r][3]);
+                if (a.uT && act)
+                    *reinterpret_cast<float4 *>(a.uT + (size_t)sample * nn + off + (size_t)(4 * b + r) * n) =
+                        make_float4(u[b][r][0], u[b][r][1], u[b][r][2], u[b][r][3]);
+            }
+            if (act) red[(strip * NB + b) * L + cc] = part;
+        }
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            double t = 0.0;
+            if (lane < L)
+                for (int k = 0; k < L; ++k) t += red[k * L + lane];
+            for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+            if (lane == 0) {
+                const double mean = t / (double)nn;
+                if (a.ubar) a.ubar[sample] = mean;
+                if (a.ooi) a.ooi[sample] = 0.5 * (1.0 + mean);
+            }
+        }
+        __syncthreads();
+    }
+}
+
+template <int R, int NB>
+mfmc_status launch_strip(const ResidentArgs &a, int sms, cudaStream_t st) {
+    auto kern = resident_strip_kernel<R, NB>;
+    const size_t smem = strip_smem(a.n, R, NB);
+    MFMC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const int nt = 32 * strip_warps(a.n, NB);
+    int per_sm = 0;
+    MFMC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, smem));
+    const int cap = (per_sm > 0 ? per_sm : 1) * sms;
+    kern<<<a.ns < cap ? a.ns : cap, nt, smem, st>>>(a);
+    MFMC_LAUNCHED("resident_strip launch");
+    return MFMC_OK;
+}
+
+template <int R>
+mfmc_status launch_resident_strip(const ResidentArgs &a, cudaStream_t st) {
+    if (a.ns <= 0) return MFMC_OK;
+    int dev = 0, sms = 0;
+    MFMC_CUDA(cudaGetDevice(&dev));
+    MFMC_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    // NB = 1 while all of the batch's four-row strips fit at 8 warps an SM (and 16 a CTA)
+    const int w1 = strip_warps(a.n, 1);
+    if (w1 <= 16 && (long long)a.ns * w1 <= 8LL * sms) return launch_strip<R, 1>(a, sms, st);
+    return launch_strip<R, 2>(a, sms, st);
+}
+
+}  // namespace mfmc
