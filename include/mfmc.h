@@ -84,7 +84,8 @@ typedef enum {
                                   TMA chunks of whole rows; a warp takes a 128-column strip
                                   of one sample, a lane 4 columns with a ring of 2R+1
                                   accumulators, every staged row summed once per segment
-                                  (constant kernel, R in {2,4,6,8}, n % 128 == 0)  */,
+                                  (constant kernel, R in {2,4,6,8}, n % 128 == 0; AUTO also
+                                  runs it at R = 12 and 16)  */,
     MFMC_ALGO_FFT = 8          /* spectral form of the disc sum: cuFFT transforms (a library,
                                   loaded at run time) of each field, a product with the
                                   transform of the disc weights and the fused update; cost

@@ -15,7 +15,21 @@
 namespace mfmc {
 
 static std::mutex g_tune_mu;
-static std::map<std::tuple<int, int, int, int, int>, std::pair<int, int>> g_tune_cache;
+// the winner, its parameter, and the fastest TMA tile shape (-1: none ran)
+struct Tuned {
+    int algo, param, tile;
+};
+static std::map<std::tuple<int, int, int, int, int>, Tuned> g_tune_cache;
+
+static void apply(Model &m, const Tuned &t) {
+    m.algo = t.algo;
+    if (t.tile >= 0) m.tma_variant = t.tile;  // also for batches too short for the row kernel
+    if (t.algo == MFMC_ALGO_ROWS) {
+        m.rows_bh = t.param / 8;
+        m.rows_rx = t.param % 8;
+    }
+    m.tuned = 1;
+}
 
 mfmc_status autotune(Model &m, cudaStream_t st) {
     if (m.d.beta2 > 0.0) {  // one solver serves beta2 > 0
@@ -28,13 +42,7 @@ mfmc_status autotune(Model &m, cudaStream_t st) {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         auto it = g_tune_cache.find(key);
         if (it != g_tune_cache.end()) {
-            m.algo = it->second.first;
-            if (m.algo == MFMC_ALGO_PREFIX_TMA) m.tma_variant = it->second.second;
-            if (m.algo == MFMC_ALGO_ROWS) {
-                m.rows_bh = it->second.second / 8;
-                m.rows_rx = it->second.second % 8;
-            }
-            m.tuned = 1;
+            apply(m, it->second);
             return MFMC_OK;
         }
     }
@@ -54,6 +62,7 @@ mfmc_status autotune(Model &m, cudaStream_t st) {
         }
     }
     std::pair<int, int> best = cands.empty() ? std::make_pair((int)MFMC_ALGO_DIRECT, 0) : cands[0];
+    int tile = -1;
     if (cands.size() > 1) {
         const size_t nn = (size_t)m.d.n * m.d.n;
         const size_t ns = std::max<size_t>(8, std::min<size_t>(1216, (size_t)(64u << 20) / nn));
@@ -71,7 +80,7 @@ mfmc_status autotune(Model &m, cudaStream_t st) {
         if (e == cudaSuccess) e = cudaEventCreate(&e1);
         if (e != cudaSuccess) s = cuda_fail(e, "autotune setup");
         if (s == MFMC_OK) s = launch_coefficients(m, nullptr, ns, coef, st);
-        float best_ms = 1e30f;
+        float best_ms = 1e30f, best_tile_ms = 1e30f;
         auto run = [&](std::pair<int, int> c) {
             if (c.first == MFMC_ALGO_PREFIX_TMA)
                 return run_solve_tma(m, 0, c.second, coef, u0, ns, steps, nullptr, nullptr, ooi, st);
@@ -106,6 +115,10 @@ mfmc_status autotune(Model &m, cudaStream_t st) {
                 cudaEventElapsedTime(&ms, e0, e1);
                 ms_min = std::min(ms_min, ms);
             }
+            if (s == MFMC_OK && cs == MFMC_OK && a.first == MFMC_ALGO_PREFIX_TMA && ms_min < best_tile_ms) {
+                best_tile_ms = ms_min;
+                tile = a.second;
+            }
             if (s == MFMC_OK && cs == MFMC_OK && ms_min < best_ms) {
                 best_ms = ms_min;
                 best = a;
@@ -120,15 +133,10 @@ mfmc_status autotune(Model &m, cudaStream_t st) {
         if (e1) cudaEventDestroy(e1);
         if (s != MFMC_OK) return s;
     }
-    m.algo = best.first;
-    if (best.first == MFMC_ALGO_PREFIX_TMA) m.tma_variant = best.second;
-    if (best.first == MFMC_ALGO_ROWS) {
-        m.rows_bh = best.second / 8;
-        m.rows_rx = best.second % 8;
-    }
-    m.tuned = 1;
+    const Tuned t{best.first, best.second, best.first == MFMC_ALGO_PREFIX_TMA ? best.second : tile};
+    apply(m, t);
     std::lock_guard<std::mutex> lk(g_tune_mu);
-    g_tune_cache[key] = best;
+    g_tune_cache[key] = t;
     return MFMC_OK;
 }
 

@@ -219,7 +219,7 @@ mfmc_status mfmc_model_create(const mfmc_model_desc *desc, mfmc_model **out) {
             m->wsq[(size_t)dy * (R + 1) + dx] = desc->kernel == MFMC_KERNEL_CONSTANT ? 1.f : m->wtab[dx * dx + dy * dy];
     m->algo = desc->algo;
     m->tuned = 0;
-    if (m->algo != MFMC_ALGO_AUTO && !algo_supported(*m, m->algo)) {
+    if (m->algo != MFMC_ALGO_AUTO && !algo_selectable(*m, m->algo)) {
         delete m;
         return fail(MFMC_EINVAL, "algorithm %d does not support this model (R=%d, kernel=%d)", (int)desc->algo, R,
                     (int)desc->kernel);
@@ -333,8 +333,10 @@ static mfmc_status solve_impl(mfmc_model *m, int algo, const double *eps, const 
             if (s != MFMC_OK) return s;
         }
         algo = m->algo;
+        if (algo == MFMC_ALGO_ROWS && rows_batch_short(*m, ns)) algo = MFMC_ALGO_PREFIX_TMA;
+    } else if (!algo_selectable(*m, algo)) {
+        return fail(MFMC_EINVAL, "algorithm %d does not support this model", algo);
     }
-    if (!algo_supported(*m, algo)) return fail(MFMC_EINVAL, "algorithm %d does not support this model", algo);
     if (algo == MFMC_ALGO_ACTIVE_SET) return run_solve_active_set(*m, eps, u0, ns, nsteps, uT, ubar, ooi, st);
     mfmc_status s = grow(&m->coef, &m->coef_cap, ns);
     if (s != MFMC_OK) return s;
@@ -394,7 +396,7 @@ mfmc_status mfmc_solve_fields(const mfmc_model *cm, const double *eps, const flo
                               double *ubar, double *ooi, void *stream) {
     if (!cm) return fail(MFMC_EINVAL, "NULL model");
     mfmc_model *m = const_cast<mfmc_model *>(cm);
-    return solve_impl(m, m->tuned ? m->algo : (int)m->d.algo, eps, u0, ns, uT, ubar, ooi, (cudaStream_t)stream);
+    return solve_impl(m, (int)m->d.algo, eps, u0, ns, uT, ubar, ooi, (cudaStream_t)stream);
 }
 
 mfmc_status mfmc_solve_fields_algo(const mfmc_model *cm, int algo, const double *eps, const float *u0, size_t ns,
@@ -454,7 +456,7 @@ mfmc_status mfmc_solve_batch(mfmc_model *const *models, const mfmc_sample_params
         MFMC_CUDA(cudaMemcpyAsync(m->eps_tmp, ep.data(), k * sizeof(double), cudaMemcpyHostToDevice, m->stream));
         mfmc_status s = mfmc_init_fields(m, params ? pp.data() : nullptr, sd.data(), k, m->u0buf, m->stream);
         if (s != MFMC_OK) return s;
-        s = solve_impl(m, m->tuned ? m->algo : (int)m->d.algo, m->eps_tmp, m->u0buf, k, nullptr, m->resbuf + k,
+        s = solve_impl(m, (int)m->d.algo, m->eps_tmp, m->u0buf, k, nullptr, m->resbuf + k,
                        m->resbuf, m->stream, gsteps);
         if (s != MFMC_OK) return s;
         host_res[g].resize(2 * k);

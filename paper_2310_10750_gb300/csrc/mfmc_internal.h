@@ -211,6 +211,7 @@ mfmc_status run_solve_rows_core(const Model &m, int bh, int rx, const StepCoef *
 mfmc_status run_solve_rows(Model &m, int bh, int rx, const StepCoef *coef, const float *u0, size_t ns, int nsteps,
                            float *uT, double *ubar, double *ooi, cudaStream_t st);
 bool rows_supported(const Model &m, int rx);
+bool rows_batch_short(const Model &m, size_t ns);
 // The TMA pipeline with an explicit tile-shape variant (autotuner).
 mfmc_status run_solve_tma(Model &m, int kahan, int variant, const StepCoef *coef, const float *u0, size_t ns,
                           int nsteps, float *uT, double *ubar, double *ooi, cudaStream_t st);
@@ -255,6 +256,10 @@ mfmc_status run_solve_active_set(Model &m, const double *eps_dev, const float *u
                                  float *uT, double *ubar, double *ooi, cudaStream_t st);
 // Whether an algorithm can run this model.
 bool algo_supported(const Model &m, int algo);
+// Whether a caller may name it for this model: the row kernel's R = 12 and 16 are AUTO's choice only.
+inline bool algo_selectable(const Model &m, int algo) {
+    return algo_supported(m, algo) && !(algo == MFMC_ALGO_ROWS && m.R > 8);
+}
 // Autotuner: time the candidate algorithms on this model once and cache the winner.
 mfmc_status autotune(Model &m, cudaStream_t st);
 

@@ -632,9 +632,10 @@ __global__ void rows_ooi_kernel(const float *plain, const float *fieldA, const f
 // 4 so each piece is a whole number of 16-byte units).
 static bool rows_geom(const Model &m, RowsGeom *g) {
     const int n = m.d.n;
-    if (n % 128 != 0 || n > 2048) return false;
+    const RowsLauncher *L = rows_launcher(m.R);
+    if (!L || n % 128 != 0 || n / 128 > L->maxw) return false;
     g->strips = n / 128;
-    g->gs = 16 / g->strips;
+    g->gs = L->maxw / g->strips;
     g->warps = g->gs * g->strips;
     g->k = 0;
     for (int k = 1; k <= 64; ++k)
@@ -643,8 +644,6 @@ static bool rows_geom(const Model &m, RowsGeom *g) {
             break;
         }
     if (g->k == 0) return false;
-    const RowsLauncher *L = rows_launcher(m.R);
-    if (!L) return false;
     g->stage_floats = g->gs * L->ch * n;
     g->smem = (size_t)L->nstg * g->stage_floats * sizeof(float) + 128;
     return g->smem <= 227 * 1024;
@@ -693,12 +692,28 @@ mfmc_status rows_alloc_buffers(const Model &m, int bh, size_t ns, TmaBuffers *b,
     return encode_rows_maps(b, m, g, L->ch);
 }
 
-// The row-streaming kernel: constant kernel, periodic lattice, integer R <= 8, 128-column strips
-// (n % 128 == 0, n <= 2048), four columns per thread.
+// The row-streaming kernel: constant kernel, periodic lattice, integer R, 128-column strips (at most
+// one CTA's warps of them a row), four columns per thread.
 bool rows_supported(const Model &m, int rx) {
     RowsGeom g;
     return m.d.kernel == MFMC_KERNEL_CONSTANT && m.d.bc == MFMC_BC_PERIODIC && m.integer_R && rx == 4 &&
            rows_launcher(m.R) != nullptr && rows_geom(m, &g);
+}
+
+// Whether a batch is too short for the row-streaming kernel: a CTA then walks 2R halo rows for few
+// rows of its own, and the tile kernel (bit-identical fields) is faster.  Measured per step, row
+// kernel against the best tile shape: 256^2, R = 8, 64 samples (1.7 R rows a CTA) 26.3 and 14.9
+// us, 128 samples (3.4 R) 27.9 and 23.7, 192 (5 R) 28.6 and 36.0; 512^2, R = 16, 32 samples (3.4 R)
+// 42.4 and 41.7, 64 (6.7 R) 57.1 and 73.4; 256^2, R = 4, 64 samples (3.4 R) 14.0 and 11.0, 128
+// (6.7 R) 15.9 and 17.3.
+bool rows_batch_short(const Model &m, size_t ns) {
+    RowsGeom g;
+    int dev = 0, sms = 0;
+    if (!rows_geom(m, &g) || cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return false;
+    const double rows = (double)((ns + g.gs - 1) / g.gs) * m.d.n;
+    return rows < 4.0 * m.R * sms;
 }
 
 mfmc_status run_solve_rows_core(const Model &m, int bh, int rx, const StepCoef *coef, const float *u0, size_t ns,

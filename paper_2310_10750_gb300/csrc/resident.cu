@@ -1,7 +1,7 @@
 // Resident kernels (the whole solve of a sample on chip): the strip form for R <= 4, the
 // shared-memory form for R = 5, 6, 8.
 #include "resident_strip.cuh"
-#include "rows_step.cuh"
+#include "tma_step.cuh"
 
 namespace mfmc {
 
@@ -38,14 +38,6 @@ const TmaLauncher *tma_launcher(int R) {
     for (auto g : groups)
         if (const TmaLauncher *t = g(R)) return t;
     return nullptr;
-}
-
-const RowsLauncher *rows_launcher_a(int R);
-const RowsLauncher *rows_launcher_b(int R);
-
-const RowsLauncher *rows_launcher(int R) {
-    if (const RowsLauncher *r = rows_launcher_a(R)) return r;
-    return rows_launcher_b(R);
 }
 
 const TileLauncher *tile_launcher(int R) {

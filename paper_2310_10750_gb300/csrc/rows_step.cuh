@@ -1,6 +1,6 @@
-// Row-streaming step kernel (constant kernel, periodic lattice, R <= 8, n % 128 == 0, n <= 2048).
+// Row-streaming step kernel (constant kernel, periodic lattice, R in {2, 4, 6, 8, 12, 16}, n % 128 == 0).
 //
-// A CTA of 16 warps (fewer when 16 is no multiple of n / 128) streams whole rows of GS
+// A CTA of MAXW warps (fewer when MAXW is no multiple of n / 128) streams whole rows of GS
 // consecutive samples down a range of rows: warp w takes the 128-column strip w % (n / 128) of
 // sample w / (n / 128) of its group, lane l the strip's columns 4l .. 4l+3.  The batch's rows,
 // ordered by (sample group, row), are split over the CTAs so that every CTA walks about as many
@@ -20,12 +20,14 @@
 // the same rows.
 //
 // From each staged row a lane forms its window's centre sums and one segment sum per distinct
-// disc-row half-width, and adds each to the 2R + 1 output rows that the row touches; the
-// accumulators (packed FP32 pairs) form a ring of 2R + 1 slots, so every staged row is summed
-// once per segment.  After staged row q the output row q - 2R is complete and is finished at
-// once (update, projection, store).  The row loop is unrolled by the ring period 2R + 1, which
-// keeps every slot index static.  The OoI is reduced afterwards from the final fields
-// (rows_ooi_kernel), so it does not depend on how the rows were split.
+// disc-row half-width, and adds them to the 2R + 1 output rows that the row touches.  The
+// accumulators (packed FP32 pairs) shift by one output row per staged row, and the shift is the
+// add itself, acc[k] = acc[k + 1] + h, so the row loop is one short body.  (A ring of 2R + 1 static
+// slots, unrolled by its period, is as fast at R = 8, 58.2 against 57.9 us a step of 512 samples of
+// 256^2, but at R = 16 its 33 rows of code miss the instruction cache: 1.92 us a sample-step of
+// 512^2 against 0.84, the tile kernel 1.14.)  After staged row q the output row q - 2R is complete and is finished at once (update, projection, store).  The OoI is
+// reduced afterwards from the final fields (rows_ooi_kernel), so it does not depend on how the
+// rows were split.
 //
 // Consecutive steps are launched as programmatic dependents: a step's CTAs set up their
 // barriers and walk while the previous step drains, and wait for its completion
@@ -62,10 +64,10 @@ struct RowsCfg {
     // a stage is refilled (with the chunk after the next) once no row of it is read again: the
     // oldest row still read is the centre row R rows back, so 2 + ceil(R / CH) stages suffice
     static constexpr int NSTG = 2 + (R + CH - 1) / CH;
-    // accumulator ring slots: the 2R + 1 output rows a staged row touches (larger rings that
-    // are multiples of CH would make chunk boundaries static but spill registers)
-    static constexpr int S = 2 * R + 1;
-    static constexpr int MAXW = 16;                      // warps per CTA at most
+    // rows per pass of the row loop, where the registers allow two (R = 16: 0.92 -> 0.84 us a
+    // sample-step of 512^2; at R = 8 two rows spill at 128 registers, 57.9 -> 74.1 us a step)
+    static constexpr int UNROLL = R > 12 ? 2 : 1;
+    static constexpr int MAXW = R > 12 ? 8 : (R > 8 ? 12 : 16);  // warps per CTA at most (255, 168 or 128 registers)
     static constexpr int MAXG = 4;                       // warp groups per CTA at most
 };
 
@@ -204,17 +206,11 @@ struct RowsSeg {
     const float *win0;   // the lane's window start (column x - R4, unwrapped) in its sample's first row of stage 0
     int wd[NQ];          // per float4 of the window: 0, or +-n where it crosses column 0 or n (never at QC)
     int bid, bthreads;   // the warp group's named barrier and its threads
-    bool leader;         // the group's first thread: walks the segments
     int tig, gw;         // the thread's index in its group, the group's warps
-    int kseg;            // index of the current segment (its slot: kseg mod 3)
-    int g0;              // stream index of the segment's first chunk
-    int nrows;           // rows walked: len + 2R
     float *out;          // the next output row's four values (rows advance by n)
-    unsigned flags;
+    int emit0;           // staged row of the segment from which output rows are finished (2R; never when inactive)
     float2 nc0, c1, c2;  // step coefficients (-c0, c1, c2) in both halves of a pair
 };
-
-enum : unsigned { kRowsActive = 1u };
 
 // The window of a lane in a staged row: WIN values from rowp, the float4s that cross a periodic
 // seam taken n columns away in the same row, then the centre sums.
@@ -246,119 +242,40 @@ __device__ __forceinline__ void rows_emit(const RowsSeg<R> &sg, float4 uc, float
                     fminf(1.f, fmaxf(-1.f, v23.y)));
 }
 
+// Staged row (window win) added to the accumulators: acc[k] holds output row q - R + k after row q.
+// The sums of output row y are added for rows y - R .. y + R in that order whatever the split.
 template <int R>
-struct RowsAcc {
-    float2 acc[RowsCfg<R>::S][2];  // slot j mod S: output row j (at most 2R + 1 live at a time)
-    const float *rp, *cp;          // the lane's window in the staged row, its centre R rows back
-    int cst;                       // stage of the centre row's chunk
-};
-
-__device__ __forceinline__ constexpr int rows_mod(int a, int m) { return ((a % m) + m) % m; }
-
-template <int R>
-struct RowsPlan {
-    static constexpr DiscClasses<R> cls{};
-    __host__ __device__ static constexpr bool serves(int dy, int c) { return cls.of[dy < 0 ? -dy : dy] == c; }
-};
-
-// Adds the class-c segment sums of staged row (ring position K) to every ring slot that the
-// class serves: dy with cls.of[|dy|] == c, output row q - R - dy in slot (K - R - dy) mod S.
-// The output row's first staged row (dy = -R) starts its slot.
-template <int R, int K, int c, int... D>
-__device__ __forceinline__ void rows_class(RowsAcc<R> &t, const RowWin<R> &win, std::integer_sequence<int, D...>) {
-    float h[4];
-    class_sums<R, RowsPlan<R>::cls.width[c]>(win, h);
-    const float2 h01 = make_float2(h[0], h[1]), h23 = make_float2(h[2], h[3]);
-    auto add = [&](auto dc) {
-        constexpr int dy = decltype(dc)::value - R;
-        if constexpr (RowsPlan<R>::serves(dy, c)) {
-            constexpr int slot = rows_mod(K - R - dy, RowsCfg<R>::S);
-            if constexpr (dy == -R) {
-                t.acc[slot][0] = h01;
-                t.acc[slot][1] = h23;
-            } else {
-                t.acc[slot][0] = __fadd2_rn(t.acc[slot][0], h01);
-                t.acc[slot][1] = __fadd2_rn(t.acc[slot][1], h23);
-            }
+__device__ __forceinline__ void rows_add(float2 (&acc)[2 * R + 1][2], const RowWin<R> &win) {
+    constexpr DiscClasses<R> cls{};
+    float2 h[R + 1][2];
+#pragma unroll
+    for (int c = cls.count - 1; c >= 0; --c) {
+        const int hw = cls.width[c];
+        constexpr int M = RowWin<R>::M, R4 = RowWin<R>::R4;
+        float t[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int b = i + R - hw, e = i + R + hw + 1;
+            t[i] = hw == 0 ? win.v[R4 + i]
+                           : (b >= M ? win.p[e] - win.p[b] : (e <= M ? win.p[b] - win.p[e] : win.p[e] + win.p[b]));
         }
-    };
-    (add(std::integral_constant<int, D>{}), ...);
-}
-
-template <int R, int K, int... Cs>
-__device__ __forceinline__ void rows_classes(RowsAcc<R> &t, const RowWin<R> &win, std::integer_sequence<int, Cs...>) {
-    (rows_class<R, K, Cs>(t, win, std::make_integer_sequence<int, 2 * R + 1>{}), ...);
-}
-
-// Staged row q = q0 + K of the segment (q0 a multiple of S, K static: the ring position).
-// Returns false when a chunk wait ran out of its bound.
-template <int R, int K>
-__device__ __forceinline__ bool rows_row(RowsAcc<R> &t, const RowsArgs &a, RowsSeg<R> &sg, int q0, RowsShared &sh,
-                                         const CUtensorMap *map, const CUtensorMap *map1, float *ring,
-                                         uint64_t *bar) {
-    using C = RowsCfg<R>;
-    const int q = q0 + K;
-    t.rp += a.pitch;
-    t.cp += a.pitch;
-    if (q % C::CH == 0) {
-        const int g = sg.g0 + q / C::CH;
-        const int st = g % C::NSTG;
-        t.rp = sg.win0 + st * a.stage_floats;
-        long long spins = 0;
-        bool ok = true;
-        while (!mbar_try_wait(&bar[st], (uint32_t)((g / C::NSTG) & 1)))
-            if (++spins > kWaitLimit) {
-                ok = false;
-                break;
-            }
-        // every thread of the group is past the rows of the stage that the next copy overwrites
-        if (!group_sync_and(sg.bid, sg.bthreads, ok)) return false;
-        // the copy is issued by lane 0 of warp g mod gw of the group: each warp carries the
-        // issue's extra work once every gw chunks, so no warp lags at every barrier
-        if (sg.tig == 32 * (g % sg.gw)) {
-            // at a segment's first chunk every warp has left the segment before it: its slot
-            // takes the segment after the next
-            if (q == 0 && sg.kseg > 0) sh.seg[(sg.kseg + 2) % 3] = sh.it.next(a);
-            rows_issue<R>(a, sh, map, map1, ring, bar);
-        }
+        h[c][0] = make_float2(t[0], t[1]);
+        h[c][1] = make_float2(t[2], t[3]);
     }
-    // the centre row q - R enters a new chunk: the stage after the previous centre chunk's
-    if ((R % C::CH == 0 ? q % C::CH == 0 : (q - R) % C::CH == 0) && q >= R) {
-        t.cst = t.cst + 1 == C::NSTG ? 0 : t.cst + 1;
-        t.cp = sg.win0 + t.cst * a.stage_floats + C::R4;
+    // ascending k: every old value is read before its register is written
+#pragma unroll
+    for (int k = 0; k < 2 * R; ++k) {
+        const int c = cls.of[k < R ? R - k : k - R];
+        acc[k][0] = __fadd2_rn(acc[k + 1][0], h[c][0]);
+        acc[k][1] = __fadd2_rn(acc[k + 1][1], h[c][1]);
     }
-    RowWin<R> win;
-    rows_window<R>(t.rp, sg, win);
-    rows_classes<R, K>(t, win, std::make_integer_sequence<int, RowsPlan<R>::cls.count>{});
-    if (q >= 2 * R) {  // output row q - 2R is complete
-        if (opaque_u32(sg.flags) & kRowsActive) {
-            constexpr int slot = rows_mod(K - 2 * R, C::S);
-            const float4 uc = *reinterpret_cast<const float4 *>(t.cp);  // its centre row, q - R
-            rows_emit<R>(sg, uc, t.acc[slot][0], t.acc[slot][1]);
-        }
-        sg.out += a.t.n;
-    }
-    return true;
+    acc[2 * R][0] = h[cls.of[R]][0];
+    acc[2 * R][1] = h[cls.of[R]][1];
 }
 
-template <int R, int... Ks>
-__device__ __forceinline__ bool rows_block(RowsAcc<R> &t, const RowsArgs &a, RowsSeg<R> &sg, int q0,
-                                           RowsShared &sh, const CUtensorMap *map, const CUtensorMap *map1,
-                                           float *ring, uint64_t *bar, int *gfail, std::integer_sequence<int, Ks...>) {
-    using C = RowsCfg<R>;
-    bool ok = true;
-    auto one = [&](auto kc) {
-        constexpr int K = decltype(kc)::value;
-        if (ok && q0 + K < sg.nrows) {
-            ok = rows_row<R, K>(t, a, sg, q0, sh, map, map1, ring, bar);
-            if (!ok) *gfail = sg.g0 + (q0 + K) / C::CH;
-        }
-    };
-    (one(std::integral_constant<int, Ks>{}), ...);
-    return ok;
-}
-
-template <int R>
+// PITCH: floats from one staged row to the next when they are fixed (MAXW strips of 128: every row
+// and centre address is then a register and a constant), 0: a.pitch.
+template <int R, int PITCH>
 __global__ void __launch_bounds__(RowsCfg<R>::MAXW * 32, 1)
     step_rows_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap map1,
                      const __grid_constant__ RowsArgs a) {
@@ -391,11 +308,10 @@ __global__ void __launch_bounds__(RowsCfg<R>::MAXW * 32, 1)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (leader) rows_issue<R>(a, sh, &map, &map1, ring, bar);
     __syncthreads();
-    RowsAcc<R> t;
-#pragma unroll
-    for (int k = 0; k < C::S; ++k) t.acc[k][0] = t.acc[k][1] = make_float2(0.f, 0.f);
 
     const int n = a.t.n, x = 128 * strip + 4 * lane;
+    const int pitch = PITCH > 0 ? PITCH : a.pitch, stage_floats = C::CH * pitch;
+    constexpr int UNROLL = PITCH > 0 ? C::UNROLL : 1;
     RowsSeg<R> sg;
     sg.win0 = ring + sl * n + x - C::R4;
 #pragma unroll
@@ -405,46 +321,88 @@ __global__ void __launch_bounds__(RowsCfg<R>::MAXW * 32, 1)
     }
     sg.bid = 1 + gid;
     sg.bthreads = 32 * gw;
-    sg.leader = leader;
     sg.tig = threadIdx.x - 32 * gw * gid;
     sg.gw = gw;
-    sg.g0 = 0;
-    int gfail = 0;
+    float2 acc[2 * R + 1][2];
+#pragma unroll
+    for (int k = 0; k <= 2 * R; ++k) acc[k][0] = acc[k][1] = make_float2(0.f, 0.f);
+    int g = 0;  // stream index of the next chunk
     bool ok = true;
     for (int k = 0; ok; ++k) {
         // segment k's slot was filled before a barrier that every warp has passed since
         const RowsSegInfo s = sh.seg[k % 3];
         if (s.len == 0) break;
-        sg.kseg = k;
-        sg.nrows = s.len + 2 * R;
-        // the centre row q - R enters chunk 0 at q = R (rows q < R have no centre in use): start
-        // one stage before the segment's first chunk
-        t.cst = (sg.g0 + C::NSTG - 1) % C::NSTG;
-        t.rp = t.cp = sg.win0;
         {
             const int sample = a.gs * s.group + sl;
             const bool active = sample < a.ns && (a.t.steps_ps == nullptr || a.t.step <= a.t.steps_ps[sample]);
             const int smp = active ? sample : 0;
+            sg.emit0 = active ? 2 * R : 0x7fffffff;
             const StepCoef cf = a.t.coef[smp];
             sg.nc0 = make_float2(-cf.c0, -cf.c0);
             sg.c1 = make_float2(cf.c1, cf.c1);
             sg.c2 = make_float2(cf.c2, cf.c2);
-            sg.flags = active ? kRowsActive : 0u;
             sg.out = a.t.dst + (size_t)smp * n * n + (size_t)s.y0 * n + x;
         }
-        for (int q0 = 0; ok && q0 < sg.nrows; q0 += C::S)
-            ok = rows_block<R>(t, a, sg, q0, sh, &map, &map1, ring, bar, &gfail,
-                               std::make_integer_sequence<int, C::S>{});
-        sg.g0 += (sg.nrows + C::CH - 1) / C::CH;
+        const int nrows = s.len + 2 * R;
+        for (int q0 = 0; q0 < nrows; q0 += C::CH, ++g) {
+            const int st = g % C::NSTG;
+            long long spins = 0;
+            while (!mbar_try_wait(&bar[st], (uint32_t)((g / C::NSTG) & 1)))
+                if (++spins > kWaitLimit) {
+                    ok = false;
+                    break;
+                }
+            // every thread of the group is past the rows of the stage that the next copy overwrites
+            if (!group_sync_and(sg.bid, sg.bthreads, ok)) {
+                ok = false;
+                break;
+            }
+            // the copy is issued by lane 0 of warp g mod gw of the group: each warp carries the
+            // issue's extra work once every gw chunks, so no warp lags at every barrier
+            if (sg.tig == 32 * (g % sg.gw)) {
+                // at a segment's first chunk every warp has left the segment before it: its slot
+                // takes the segment after the next
+                if (q0 == 0 && k > 0) sh.seg[(k + 2) % 3] = sh.it.next(a);
+                rows_issue<R>(a, sh, &map, &map1, ring, bar);
+            }
+            const float *rp = sg.win0 + st * stage_floats;
+            // the centre row of staged row r: row r - R % CH of chunk g - R / CH, or row r + CH - R % CH
+            // of the chunk before it
+            int sa = st - R / C::CH, sb;
+            sa += sa < 0 ? C::NSTG : 0;
+            sb = sa == 0 ? C::NSTG - 1 : sa - 1;
+            const float *ca = sg.win0 + C::R4 + sa * stage_floats - R % C::CH * pitch;
+            const float *cb = sg.win0 + C::R4 + sb * stage_floats + (C::CH - R % C::CH) * pitch;
+            auto row = [&](int r) {
+                RowWin<R> win;
+                rows_window<R>(rp + r * pitch, sg, win);
+                rows_add<R>(acc, win);
+                if (q0 + r >= sg.emit0) {  // output row q - 2R is complete; its centre row is q - R
+                    const float4 uc = *reinterpret_cast<const float4 *>((r >= R % C::CH ? ca : cb) + r * pitch);
+                    rows_emit<R>(sg, uc, acc[0][0], acc[0][1]);
+                    sg.out += n;
+                }
+            };
+            if (nrows - q0 >= C::CH) {
+#pragma unroll 1
+                for (int h = 0; h < C::CH; h += UNROLL) {
+#pragma unroll
+                    for (int r = 0; r < UNROLL; ++r) row(h + r);
+                }
+            } else {
+#pragma unroll 1
+                for (int r = 0; r < nrows - q0; ++r) row(r);
+            }
+        }
     }
     if (!ok && leader) {
         // A chunk wait ran out of its bound (only a copy that never lands can cause it): report,
         // then wait, again bounded, for each copy issued and not consumed, so that none still
         // targets the ring when the CTA exits unless that wait runs out as well.
         atomicExch(a.t.status, 1);
-        for (int g = gfail; g < sh.pg; ++g) {
+        for (int j = g; j < sh.pg; ++j) {
             long long spins = 0;
-            while (!mbar_try_wait(&bar[g % C::NSTG], (uint32_t)((g / C::NSTG) & 1)) && ++spins < kWaitLimit) {
+            while (!mbar_try_wait(&bar[j % C::NSTG], (uint32_t)((j / C::NSTG) & 1)) && ++spins < kWaitLimit) {
             }
         }
     }
@@ -465,7 +423,7 @@ struct RowsGeom {
 };
 
 struct RowsLauncher {
-    int ch, nstg;
+    int ch, nstg, maxw;
     // pdl: launch as a programmatic dependent of the previous kernel in the stream (a step)
     mfmc_status (*fn)(const CUtensorMap &map, const CUtensorMap &map1, const RowsArgs &, int grid, int threads,
                       size_t smem, bool pdl, cudaStream_t);
@@ -475,7 +433,7 @@ struct RowsLauncher {
 template <int R>
 mfmc_status launch_rows(const CUtensorMap &map, const CUtensorMap &map1, const RowsArgs &a, int grid, int threads,
                         size_t smem, bool pdl, cudaStream_t st) {
-    auto kern = step_rows_kernel<R>;
+    auto kern = a.pitch == RowsCfg<R>::MAXW * 128 ? step_rows_kernel<R, RowsCfg<R>::MAXW * 128> : step_rows_kernel<R, 0>;
     MFMC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
@@ -494,7 +452,7 @@ mfmc_status launch_rows(const CUtensorMap &map, const CUtensorMap &map1, const R
 
 template <int R>
 int rows_blocks_per_sm(int threads, size_t smem) {
-    auto kern = step_rows_kernel<R>;
+    auto kern = step_rows_kernel<R, 0>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int per = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, threads, smem);
@@ -507,6 +465,7 @@ RowsLauncher make_rows_launcher() {
     RowsLauncher L;
     L.ch = RowsCfg<R>::CH;
     L.nstg = RowsCfg<R>::NSTG;
+    L.maxw = RowsCfg<R>::MAXW;
     L.fn = &launch_rows<R>;
     L.blocks_per_sm = &rows_blocks_per_sm<R>;
     return L;
