@@ -30,6 +30,8 @@ namespace mfmc {
 
 namespace {
 
+constexpr int AT_NU_COARSE = 8;  // coarsest sweeps (16, as the fallback kernel has: no CG iteration fewer)
+
 template <int N>
 struct AtCfg {
     static constexpr int CW = N == 64 ? 2 : 4;      // columns per lane
@@ -297,7 +299,7 @@ __device__ __forceinline__ void tail_coarsest(const TailLanes<n> &p, const float
         v[y] = w[y] * f[y];
     }
 #pragma unroll 1
-    for (int k = 2; k <= AS_NU_COARSE; ++k) tail_sweep<n>(p, f, w, v, tb2);
+    for (int k = 2; k <= AT_NU_COARSE; ++k) tail_sweep<n>(p, f, w, v, tb2);
 }
 
 // One cycle from f to v (shared memory, n x n) by one warp; d: the diagonals.
@@ -619,7 +621,11 @@ __global__ void __launch_bounds__(AtCfg<N>::NT, MINB) active_set_tile_kernel(con
             for (int y = 0; y < RW; ++y)
 #pragma unroll
                 for (int c = 0; c < CW; ++c) f[y][c] *= sc;
-            // CG on J d = f from d = 0, preconditioned by one V-cycle
+            // CG on J d = f from d = 0, preconditioned by one V-cycle, to a residual that matches what the
+            // correction can be worth: while the active set still moves it limits the next residual, not
+            // the solve, and on a settled set the next residual is this one times the tolerance (1e-5
+            // throughout: 33.1 CG iterations a step of 128^2 samples, now 26.1)
+            const float rtol = it == 1 ? 3e-2f : (changed ? 1e-3f : 1e-6f);
             float rz = 0.0f;
             for (int k = 1;; ++k) {
                 float v[RW][CW];
@@ -683,7 +689,7 @@ __global__ void __launch_bounds__(AtCfg<N>::NT, MINB) active_set_tile_kernel(con
                     }
                 }
                 rmax = t.max(rmax);
-                if (rmax <= AS_CG_RTOL || !(pq > 0.0f) || !(rz > 0.0f) || k >= a.cg_max) {
+                if (rmax <= rtol || !(pq > 0.0f) || !(rz > 0.0f) || k >= a.cg_max) {
                     n_cg += k;
                     break;
                 }
@@ -760,8 +766,8 @@ bool as_tile_supported(int n) { return n == 64 || n == 88 || n == 128; }
 
 mfmc_status launch_active_set_tile(const AsTileArgs &a, int n, unsigned grid, cudaStream_t st) {
     switch (n) {
-        case 64: return at_launch<64, 3>(a, grid, st);
-        case 88: return at_launch<88, 1>(a, grid, st);
+        case 64: return at_launch<64, 4>(a, grid, st);
+        case 88: return at_launch<88, 2>(a, grid, st);
         case 128: return at_launch<128, 1>(a, grid, st);
         default: return fail(MFMC_EINVAL, "no on-chip active-set kernel for n = %d", n);
     }
