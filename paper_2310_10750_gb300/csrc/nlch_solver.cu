@@ -10,6 +10,7 @@
 
 #include <mutex>
 
+#include "resident_cluster.cuh"
 #include "rows_step.cuh"
 
 namespace mfmc {
@@ -354,6 +355,7 @@ bool algo_supported(const Model &m, int algo) {
         case MFMC_ALGO_PREFIX_TMA: return constant && tma_launcher(m.R) != nullptr;
         case MFMC_ALGO_ROWS: return constant && rows_supported(m, 4);
         case MFMC_ALGO_RESIDENT: {
+            if (constant && resident_cluster_shape(m.d.n, m.R)) return true;
             if (!constant || resident_launcher(m.R) == nullptr) return false;
             const int nt = resident_threads(m.d.n);
             return m.d.n % 4 == 0 && (m.d.n * m.d.n) % (4 * RES_RY) == 0 && nt >= 1 && nt <= 256 &&
@@ -824,6 +826,7 @@ mfmc_status run_resident_steps(const Model &m, const StepCoef *coef, const float
     a.n = m.d.n;
     a.ns = (int)ns;
     a.nsteps = nsteps;
+    if (resident_cluster_shape(a.n, m.R)) return launch_resident_cluster(m.R, a, st);
     ResidentFn f = resident_launcher(m.R);
     if (!f) return fail(MFMC_EINVAL, "no resident kernel for R = %d", m.R);
     return f(a, st);
