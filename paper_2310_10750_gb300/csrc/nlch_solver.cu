@@ -134,6 +134,44 @@ __global__ void __launch_bounds__(IC_NT) smoothed_ic_kernel(int n, double amp, i
     }
 }
 
+// The nuclei IC, separable: exp(-36 (dx^2 + dy^2)) = exp(-36 dx^2) exp(-36 dy^2), so a CTA of NU_ROWS
+// rows of one sample evaluates 4 (n + NU_ROWS) exponentials where init_fields_kernel evaluates four
+// a node, which at two FP64 lanes a clock an SM took most of 1 ms for 64 samples of 256^2 (the
+// whole call from seeds to OoIs, 500 steps: 4.67 -> 3.72 ms).  The
+// product of two rounded exponentials is within 2 FP64 ulps, far below the FP32 rounding.
+constexpr int NU_ROWS = 32, NU_NT = 256;
+
+// exp(-36 d^2) for the minimum-image distance d of lattice coordinate i from c
+__device__ __forceinline__ double nuclei_factor(int i, double h, double c) {
+    double d = __dsub_rn(__dmul_rn((double)i, h), c);
+    d = __dsub_rn(d, floor(__dadd_rn(d, 0.5)));
+    return exp(__dmul_rn(-36.0, __dmul_rn(d, d)));
+}
+
+__global__ void __launch_bounds__(NU_NT) nuclei_ic_kernel(int n, const double *theta, size_t s0, float *u0) {
+    extern __shared__ double nu_ex[];  // [4][n] factors along x, times the depths mu
+    __shared__ double ey[4][NU_ROWS];
+    const size_t smp = s0 + blockIdx.y;
+    const int y0 = blockIdx.x * NU_ROWS, rows = min(NU_ROWS, n - y0);
+    const double *th = theta + smp * 12;
+    const double cx[4] = {0.25, 0.75, 0.5, 0.5}, cy[4] = {0.5, 0.5, 0.25, 0.75}, h = 1.0 / n;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        for (int i = threadIdx.x; i < n; i += NU_NT)
+            nu_ex[k * n + i] = __dmul_rn(th[k], nuclei_factor(i, h, __dadd_rn(cx[k], th[4 + 2 * k])));
+        if ((int)threadIdx.x < rows) ey[k][threadIdx.x] = nuclei_factor(y0 + threadIdx.x, h, __dadd_rn(cy[k], th[5 + 2 * k]));
+    }
+    __syncthreads();
+    float *out = u0 + smp * (size_t)n * n + (size_t)y0 * n;
+    for (int i = threadIdx.x; i < rows * n; i += NU_NT) {
+        const int y = i / n, x = i - y * n;
+        double s = 0.0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) s = fma(nu_ex[k * n + x], ey[k][y], s);
+        out[i] = (float)clip1(fma(-2.0, s, 1.0));
+    }
+}
+
 mfmc_status launch_init_fields(const Model &m, const uint64_t *seeds_dev, const double *theta_dev,
                                size_t ns, float *u0, cudaStream_t st) {
     if (ns == 0) return MFMC_OK;
@@ -150,6 +188,15 @@ mfmc_status launch_init_fields(const Model &m, const uint64_t *seeds_dev, const 
                                                                              seeds_dev, o, u0);
         }
         MFMC_LAUNCHED("nlch_solver launch 1 (tiled)");
+        return MFMC_OK;
+    }
+    if (m.d.ic == MFMC_IC_NUCLEI && m.d.n <= 1024) {  // (the factors of larger lattices do not fit 48 KB)
+        for (size_t o = 0; o < ns; o += 65535) {
+            const unsigned gy = (unsigned)std::min<size_t>(65535, ns - o);
+            nuclei_ic_kernel<<<dim3((unsigned)((m.d.n + NU_ROWS - 1) / NU_ROWS), gy), NU_NT,
+                               (size_t)4 * m.d.n * sizeof(double), st>>>(m.d.n, theta_dev, o, u0);
+        }
+        MFMC_LAUNCHED("nlch_solver launch 1 (nuclei)");
         return MFMC_OK;
     }
     init_fields_kernel<<<(unsigned)blocks, block, 0, st>>>(m.d.n, (int)m.d.ic, m.d.ic_amp, base_n, seeds_dev,
