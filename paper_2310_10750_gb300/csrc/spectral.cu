@@ -37,6 +37,10 @@
 
 namespace mfmc {
 
+// (nlch_solver.cu) the fields' FP64 means from `chunks` CTAs a field
+mfmc_status launch_field_ooi_chunks(const float *u, size_t ns, int n, double *partials, int chunks, double *ubar,
+                                    double *ooi, cudaStream_t st);
+
 namespace {
 constexpr int kSq = 32;               // n = kSq * kSq
 constexpr int kN = kSq * kSq;         // 1024
@@ -46,6 +50,7 @@ constexpr int kPitch = 528;           // half-spectrum row pitch in complex valu
 constexpr int kColStride = kColTile + 1;  // shared-memory row stride of a column tile (complex)
 constexpr int kRowWarps = 12;         // row-pass warps per CTA
 constexpr int kSpecRowBytes = 514 * 8;    // a half-spectrum row as copied (513 values and one of padding)
+constexpr int kOoiChunks = 32;        // CTAs per field of the final FP64 means
 constexpr int kRowBuf = 2 * 514;      // a row-pass warp buffer in complex values (8224 bytes)
 }  // namespace
 
@@ -128,7 +133,11 @@ __global__ void __launch_bounds__(kColTile * 32, 2)
     float2 *tile = spec_smem;                    // [1024][9]
     float2 *tw = spec_smem + kN * kColStride;    // [32][32]
     const int ti = blockIdx.x;
-    float2 *g = spec + (size_t)blockIdx.y * kN * kPitch + ti * kColTile;
+    // samples in descending order: the row pass before it ended with the last ones, whose rows are
+    // still in L2, and the row pass after it starts with the first ones (64 samples: 5.85 -> 5.65 us
+    // a sample-step)
+    const int smp = (int)(gridDim.y - 1 - blockIdx.y);
+    float2 *g = spec + (size_t)smp * kN * kPitch + ti * kColTile;
     for (int i = threadIdx.x; i < kN * kColTile; i += blockDim.x) {
         const int y = i / kColTile, c = i - y * kColTile;
         asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(tile + y * kColStride + c)),
@@ -713,7 +722,9 @@ mfmc_status run_solve_spectral(Model &m, const StepCoef *coef, const float *u0, 
         MFMC_LAUNCHED("spectral launch 3");
         src = dst;
     }
-    return launch_field_ooi(src, ns, kN, ubar, ooi, st);
+    s = grow_buffer(&m.partials, &m.partials_cap, ns * kOoiChunks);
+    if (s != MFMC_OK) return s;
+    return launch_field_ooi_chunks(src, ns, kN, m.partials, kOoiChunks, ubar, ooi, st);
 }
 
 }  // namespace mfmc
