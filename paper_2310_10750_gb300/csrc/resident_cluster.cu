@@ -9,9 +9,11 @@
 // rows.  So no row is summed twice, where the row-streaming kernel walks 2R halo rows per range
 // (half its walk and more for a batch of 64 samples) and streams the fields through HBM.
 //
-// A step has two cluster barriers: partial sums written before they are read (waited for at once),
-// and read before the next step writes them (the wait comes after the next step's first row).  The
-// two column strips of a row (n = 256) meet at a 64-thread barrier once their row block is updated.
+// A step has one cluster barrier, between the partial sums' writes and reads, and one of the CTA,
+// between their reads and the next step's writes; the buffers that another CTA writes alternate, so
+// that a write can only meet the reads of two steps before, which the cluster barrier of the step
+// between has ordered.  The two column strips of a row (n = 256) meet at a 64-thread barrier once
+// their row block is updated.
 //
 // What bounds it: shared memory, 44 wavefronts a row of 128 columns (window 20, partial sums 16,
 // field 8): 5.6 K cycles a step of 64 x 256 points on an SM, the FMA pipe 4.0 K.
@@ -36,7 +38,10 @@ struct RcCfg {
     static constexpr int CL = N / ROWS;                 // CTAs per sample
     static constexpr int FIELD = ROWS * N;              // floats
     static constexpr int IN = RC_WARPS * 2 * R * 128;   // floats: per warp R rows from above, R from below
-    static constexpr size_t SMEM = (size_t)(FIELD + IN) * sizeof(float);
+    // the buffers that another CTA writes (top strip's "above", bottom strip's "below") alternate
+    // between IN and this second copy from step to step
+    static constexpr int FAR = CL > 1 ? 2 * XS * R * 128 : 0;  // floats: [above, below][column strip][R]
+    static constexpr size_t SMEM = (size_t)(FIELD + IN + FAR) * sizeof(float);
 };
 
 __device__ __forceinline__ uint32_t rc_map(uint32_t addr, uint32_t rank) {
@@ -49,16 +54,15 @@ __device__ __forceinline__ void rc_st_remote(uint32_t addr, float2 a, float2 b) 
                  : "memory");
 }
 
+// Barrier of the sample's CTAs.
 template <int CL>
-__device__ __forceinline__ void rc_arrive() {
-    if constexpr (CL > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-}
-template <int CL>
-__device__ __forceinline__ void rc_wait() {
-    if constexpr (CL > 1)
+__device__ __forceinline__ void rc_sync() {
+    if constexpr (CL > 1) {
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    else
+    } else {
         __syncthreads();
+    }
 }
 
 template <int N, int R>
@@ -86,9 +90,12 @@ __global__ void __launch_bounds__(RC_NT, 1) resident_cluster_kernel(ResidentArgs
     const bool up_out = strip == 0, dn_out = strip == K::STRIPS - 1;
     const int up_warp = (up_out ? K::STRIPS - 1 : strip - 1) * K::XS + xs, dn_warp = (dn_out ? 0 : strip + 1) * K::XS + xs;
     float4 *const up_dst = in + ((up_warp * 2 + 1) * R) * 32 + lane, *const dn_dst = in + ((dn_warp * 2 + 0) * R) * 32 + lane;
-    const uint32_t up_addr = rc_map(smem_u32(up_dst), CL > 1 ? (rank + CL - 1) % CL : 0);
-    const uint32_t dn_addr = rc_map(smem_u32(dn_dst), CL > 1 ? (rank + 1) % CL : 0);
+    float4 *const far = reinterpret_cast<float4 *>(rc_smem + K::FIELD + K::IN) + xs * R * 32 + lane;  // [above, below]
+    const uint32_t up_rank = CL > 1 ? (rank + CL - 1) % CL : 0, dn_rank = CL > 1 ? (rank + 1) % CL : 0;
+    const uint32_t up_addr[2] = {rc_map(smem_u32(up_dst), up_rank), rc_map(smem_u32(far + K::XS * R * 32), up_rank)};
+    const uint32_t dn_addr[2] = {rc_map(smem_u32(dn_dst), dn_rank), rc_map(smem_u32(far), dn_rank)};
     const bool up_far = CL > 1 && up_out, dn_far = CL > 1 && dn_out;
+    const bool dn_far_in = up_far, up_far_in = dn_far;  // the top strip's "above" and the bottom's "below" come from afar
     const float4 *const from_up = in + ((warp * 2 + 0) * R) * 32 + lane, *const from_dn = in + ((warp * 2 + 1) * R) * 32 + lane;
     const size_t nn = (size_t)N * N, off = (size_t)(rank * K::ROWS + strip * RC_ROWS) * N + x;
 
@@ -107,10 +114,11 @@ __global__ void __launch_bounds__(RC_NT, 1) resident_cluster_kernel(ResidentArgs
         const StepCoef cf = a.coef[sample];
         const float2 nc0 = make_float2(-cf.c0, -cf.c0), c1 = make_float2(cf.c1, cf.c1), c2 = make_float2(cf.c2, cf.c2);
         const int nsteps = a.steps_ps ? a.steps_ps[sample] : a.nsteps;
-        rc_arrive<CL>();  // the buffers are free (nobody reads them before the first step's barrier)
+        rc_sync<CL>();  // every CTA of the cluster runs and has left the sample before
         pair_sync();
 #pragma unroll 1
         for (int step = 0; step < nsteps; ++step) {
+            const int alt = step & 1;
             float2 own[RC_ROWS][2], up[R][2], dn[R][2];
 #pragma unroll
             for (int r = 0; r < RC_ROWS; ++r) {
@@ -153,11 +161,11 @@ __global__ void __launch_bounds__(RC_NT, 1) resident_cluster_kernel(ResidentArgs
                         }
                     }
                 }
-                if (r == 0) rc_wait<CL>();  // every strip has read the last step's sums
+                if (r == 0) __syncthreads();  // every strip of the CTA has read the last step's sums
                 // output row r - R of the strip above has all of this strip's rows
                 if (r < R) {
                     if (up_far)
-                        rc_st_remote(up_addr + 512 * r, up[r < R ? r : 0][0], up[r < R ? r : 0][1]);
+                        rc_st_remote((alt ? up_addr[1] : up_addr[0]) + 512 * r, up[r < R ? r : 0][0], up[r < R ? r : 0][1]);
                     else
                         up_dst[32 * r] = make_float4(up[r < R ? r : 0][0].x, up[r < R ? r : 0][0].y,
                                                      up[r < R ? r : 0][1].x, up[r < R ? r : 0][1].y);
@@ -166,27 +174,26 @@ __global__ void __launch_bounds__(RC_NT, 1) resident_cluster_kernel(ResidentArgs
 #pragma unroll
             for (int k = 0; k < R; ++k) {
                 if (dn_far)
-                    rc_st_remote(dn_addr + 512 * k, dn[k][0], dn[k][1]);
+                    rc_st_remote((alt ? dn_addr[1] : dn_addr[0]) + 512 * k, dn[k][0], dn[k][1]);
                 else
                     dn_dst[32 * k] = make_float4(dn[k][0].x, dn[k][0].y, dn[k][1].x, dn[k][1].y);
             }
-            rc_arrive<CL>();
-            rc_wait<CL>();
+            rc_sync<CL>();
             // (own + from above) + from below
+            const float4 *const fu = dn_far_in && alt ? far : from_up, *const fd = up_far_in && alt ? far + K::XS * R * 32 : from_dn;
 #pragma unroll
             for (int y = 0; y < RC_ROWS; ++y) {
                 if (y < R) {
-                    const float4 t = from_up[32 * y];
+                    const float4 t = fu[32 * y];
                     own[y][0] = __fadd2_rn(own[y][0], make_float2(t.x, t.y));
                     own[y][1] = __fadd2_rn(own[y][1], make_float2(t.z, t.w));
                 }
                 if (y >= RC_ROWS - R) {
-                    const float4 t = from_dn[32 * (y - (RC_ROWS - R))];
+                    const float4 t = fd[32 * (y - (RC_ROWS - R))];
                     own[y][0] = __fadd2_rn(own[y][0], make_float2(t.x, t.y));
                     own[y][1] = __fadd2_rn(own[y][1], make_float2(t.z, t.w));
                 }
             }
-            rc_arrive<CL>();
 #pragma unroll
             for (int y = 0; y < RC_ROWS; ++y) {
                 float4 *p = reinterpret_cast<float4 *>(mine + y * N + x);
@@ -199,7 +206,6 @@ __global__ void __launch_bounds__(RC_NT, 1) resident_cluster_kernel(ResidentArgs
             }
             pair_sync();
         }
-        rc_wait<CL>();
         // OoI: FP64, rows then lanes then warps then CTAs in order
         double part = 0.0;
 #pragma unroll
@@ -220,8 +226,7 @@ __global__ void __launch_bounds__(RC_NT, 1) resident_cluster_kernel(ResidentArgs
             else
                 cta_sum[0] = t;
         }
-        rc_arrive<CL>();
-        rc_wait<CL>();
+        rc_sync<CL>();
         if (rank == 0 && threadIdx.x == 0) {
             double t = 0.0;
             for (int i = 0; i < CL; ++i) t += cta_sum[i];
