@@ -66,7 +66,9 @@ mfmc_status autotune(Model &m, cudaStream_t st) {
     if (cands.size() > 1) {
         const size_t nn = (size_t)m.d.n * m.d.n;
         const size_t ns = std::max<size_t>(8, std::min<size_t>(1216, (size_t)(64u << 20) / nn));
-        const int steps = std::max(1, std::min(m.d.nsteps, 16));
+        // not the model's own count: the winner is cached for every model of this lattice and horizon,
+        // and a one-step model would settle on a form that only saves the set-up of a solve
+        const int steps = 16;
         float *u0 = nullptr;
         StepCoef *coef = nullptr;
         double *ooi = nullptr;
