@@ -1,5 +1,4 @@
-// Resident kernels (the whole solve of a sample on chip): the strip form for R <= 4, the
-// shared-memory form for R = 5, 6, 8.
+// Resident kernels (the whole solve of a sample on chip) in strips, and the per-R launcher tables.
 #include "resident_strip.cuh"
 #include "tma_step.cuh"
 
@@ -11,9 +10,9 @@ ResidentFn resident_launcher(int R) {
         case 2: return &launch_resident_strip<2>;
         case 3: return &launch_resident_strip<3>;
         case 4: return &launch_resident_strip<4>;
-        case 5: return &launch_resident<5>;
-        case 6: return &launch_resident<6>;
-        case 8: return &launch_resident<8>;
+        case 5: return &launch_resident_strip<5>;
+        case 6: return &launch_resident_strip<6>;
+        case 8: return &launch_resident_strip<8>;
         default: return nullptr;
     }
 }

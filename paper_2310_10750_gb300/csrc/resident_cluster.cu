@@ -266,7 +266,7 @@ mfmc_status rc_launch(const ResidentArgs &a, cudaStream_t st) {
 
 mfmc_status launch_resident_cluster(int R, const ResidentArgs &a, cudaStream_t st) {
     if (a.ns <= 0) return MFMC_OK;
-    if (a.n == 128) return R == 6 ? rc_launch<128, 6>(a, st) : rc_launch<128, 8>(a, st);
+    if (a.n == 128) return R == 5 ? rc_launch<128, 5>(a, st) : (R == 6 ? rc_launch<128, 6>(a, st) : rc_launch<128, 8>(a, st));
     return R == 4 ? rc_launch<256, 4>(a, st) : (R == 6 ? rc_launch<256, 6>(a, st) : rc_launch<256, 8>(a, st));
 }
 

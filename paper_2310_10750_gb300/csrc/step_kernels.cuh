@@ -220,10 +220,8 @@ constexpr size_t tile_smem_bytes() {
     return (size_t)(RY * TYT + 2 * R) * (4 * TXT + 2 * ((R + 3) & ~3)) * sizeof(float);
 }
 
-// Whole field resident in shared memory for every step (one CTA per sample).  The
-// padded array holds the n x n field plus its periodic images in an R-row / R4-column
-// collar.  Each step every thread computes its 4 x RY block into registers, the block
-// synchronises, and the new values are written over the old ones and their images.
+// Arguments of the resident solves (resident_strip.cuh, resident_cluster.cu): a sample's whole field on
+// chip for every step.
 struct ResidentArgs {
     const float *u0;
     float *uT;
@@ -235,127 +233,6 @@ struct ResidentArgs {
     int ns;
     int nsteps;
 };
-
-template <int R, int RY>
-__global__ void __launch_bounds__(256) resident_kernel(ResidentArgs a) {
-    constexpr int RX = 4;
-    constexpr int R4 = (R + 3) & ~3;
-    constexpr int WIN = RX + 2 * R4;
-    constexpr DiscRows<R> disc{};
-    extern __shared__ float4 smem4[];
-    float *s = reinterpret_cast<float *>(smem4);
-    __shared__ double red[256];
-
-    const int n = a.n;
-    const int SW = n + 2 * R4;
-    const int SW4 = SW / 4;
-    const int SH = n + 2 * R;
-    const int TXT = n / 4;
-    const int tx = threadIdx.x % TXT;
-    const int ty = threadIdx.x / TXT;
-    const int ox = tx * RX;
-    const int oy = ty * RY;
-    const int nt = blockDim.x;
-    const size_t nn = (size_t)n * n;
-
-    for (int sample = blockIdx.x; sample < a.ns; sample += gridDim.x) {
-        const float *__restrict__ src = a.u0 + (size_t)sample * nn;
-        for (int idx = threadIdx.x; idx < SH * SW4; idx += nt) {
-            const int r = idx / SW4;
-            const int c4 = idx - r * SW4;
-            const int gy = wrap_idx(r - R, n);
-            const int gx = wrap_idx(4 * c4 - R4, n);
-            smem4[idx] = __ldg(reinterpret_cast<const float4 *>(src + (size_t)gy * n + gx));
-        }
-        const StepCoef cf = a.coef[sample];
-        __syncthreads();
-
-        float o[RY][RX];
-        const int nsteps = a.steps_ps ? a.steps_ps[sample] : a.nsteps;
-        for (int step = 0; step < nsteps; ++step) {
-            float acc[RY][RX];
-#pragma unroll
-            for (int j = 0; j < RY; ++j)
-#pragma unroll
-                for (int i = 0; i < RX; ++i) acc[j][i] = 0.f;
-#pragma unroll
-            for (int r = 0; r < RY + 2 * R; ++r) {
-                const float4 *rowp = reinterpret_cast<const float4 *>(s + (oy + r) * SW + ox);
-                float v[WIN];
-#pragma unroll
-                for (int q = 0; q < WIN / 4; ++q) {
-                    const float4 t = rowp[q];
-                    v[4 * q + 0] = t.x;
-                    v[4 * q + 1] = t.y;
-                    v[4 * q + 2] = t.z;
-                    v[4 * q + 3] = t.w;
-                }
-                float p[RX + 2 * R + 1];
-                p[0] = 0.f;
-#pragma unroll
-                for (int k = 0; k < RX + 2 * R; ++k) p[k + 1] = p[k] + v[R4 - R + k];
-#pragma unroll
-                for (int j = 0; j < RY; ++j) {
-                    const int dy = r - R - j;
-                    if (dy >= -R && dy <= R) {
-                        const int w = disc.w[dy < 0 ? -dy : dy];
-#pragma unroll
-                        for (int i = 0; i < RX; ++i) acc[j][i] += p[i + R + w + 1] - p[i + R - w];
-                    }
-                }
-            }
-#pragma unroll
-            for (int j = 0; j < RY; ++j) {
-                const float4 c4v = *reinterpret_cast<const float4 *>(s + (oy + j + R) * SW + ox + R4);
-                const float uc[4] = {c4v.x, c4v.y, c4v.z, c4v.w};
-#pragma unroll
-                for (int i = 0; i < RX; ++i) {
-                    const float sd = fmaf(-cf.c0, uc[i], acc[j][i]);
-                    const float v = uc[i] + fmaf(cf.c1, sd, cf.c2 * uc[i]);
-                    o[j][i] = fminf(1.f, fmaxf(-1.f, v));
-                }
-            }
-            __syncthreads();
-            // write back the block and its periodic images
-            const bool left = ox < R4, right = ox >= n - R4;
-#pragma unroll
-            for (int j = 0; j < RY; ++j) {
-                const float4 val = make_float4(o[j][0], o[j][1], o[j][2], o[j][3]);
-                const int y = oy + j;
-                const int rows[3] = {y + R, y < R ? y + R + n : -1, y >= n - R ? y + R - n : -1};
-#pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                    const int pr = rows[q];
-                    if (pr < 0) continue;
-                    float *rowb = s + pr * SW;
-                    *reinterpret_cast<float4 *>(rowb + ox + R4) = val;
-                    if (left) *reinterpret_cast<float4 *>(rowb + ox + R4 + n) = val;
-                    if (right) *reinterpret_cast<float4 *>(rowb + ox + R4 - n) = val;
-                }
-            }
-            __syncthreads();
-        }
-        // output of interest and optional final field
-        double part = 0.0;
-#pragma unroll
-        for (int j = 0; j < RY; ++j) {
-            const float4 c4v = *reinterpret_cast<const float4 *>(s + (oy + j + R) * SW + ox + R4);
-            part += ((double)c4v.x + (double)c4v.y) + ((double)c4v.z + (double)c4v.w);
-            if (a.uT)
-                *reinterpret_cast<float4 *>(a.uT + (size_t)sample * nn + (size_t)(oy + j) * n + ox) = c4v;
-        }
-        red[threadIdx.x] = part;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double t = 0.0;
-            for (int i = 0; i < nt; ++i) t += red[i];
-            const double mean = t / (double)nn;
-            if (a.ubar) a.ubar[sample] = mean;
-            if (a.ooi) a.ooi[sample] = 0.5 * (1.0 + mean);
-        }
-        __syncthreads();
-    }
-}
 
 // ----------------------------------------------------------------------------- launchers
 // Register-tiled kernel configuration per R: 64-column tiles, 4 x RY outputs per thread.
@@ -405,6 +282,9 @@ TileLauncher make_tile_launcher() {
     return L;
 }
 
+// The lattices the resident form serves: n a multiple of 16, at most 256 blocks of 4 x 16 points, the
+// field with its periodic frame within 225 KB (the frame of a form that held it in shared memory;
+// kept as the rule, so that what it accepts does not change).
 constexpr int RES_RY = 16;
 
 inline size_t resident_smem(int n, int R) {
@@ -413,24 +293,6 @@ inline size_t resident_smem(int n, int R) {
 }
 
 inline int resident_threads(int n) { return n * n / (4 * RES_RY); }
-
-template <int R>
-mfmc_status launch_resident(const ResidentArgs &a, cudaStream_t st) {
-    auto kern = resident_kernel<R, RES_RY>;
-    const size_t smem = resident_smem(a.n, R);
-    MFMC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    const int nt = resident_threads(a.n);
-    int per_sm = 0;
-    MFMC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, smem));
-    int dev = 0, sms = 0;
-    MFMC_CUDA(cudaGetDevice(&dev));
-    MFMC_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const int cap = (per_sm > 0 ? per_sm : 1) * sms;
-    const int grid = a.ns < cap ? a.ns : cap;
-    kern<<<grid > 0 ? grid : 1, nt, smem, st>>>(a);
-    MFMC_LAUNCHED("step_kernels launch 2");
-    return MFMC_OK;
-}
 
 typedef mfmc_status (*ResidentFn)(const ResidentArgs &, cudaStream_t);
 

@@ -33,10 +33,10 @@ def seeds_of(k, base):
     return np.arange(k, dtype=np.uint64) + base
 
 
-# resident strips (R <= 4): lattices from 16 (eight strips a warp) to 128 (one row a warp), with idle
+# resident strips (blocks of four rows to R = 4, of eight above): lattices from 16 (eight strips a warp) to 128 (one row a warp), with idle
 # lanes (48: two groups of 12, 96: 24 of 32, 112: 28 of 32) and idle groups
 @pytest.mark.parametrize("n,R", [(16, 1), (16, 3), (16, 4), (32, 2), (48, 4), (80, 3), (96, 1), (96, 4), (112, 2),
-                                 (128, 1), (128, 4)])
+                                 (128, 1), (128, 4), (16, 6), (32, 8), (48, 5), (64, 8), (96, 6), (112, 8)])
 @pytest.mark.parametrize("ic", [1, 2])
 def test_resident_strips(gpu_lib, n, R, ic):
     mf = gpu_lib
@@ -64,7 +64,7 @@ def test_resident_strips_do_not_depend_on_the_batch(gpu_lib, n, R, many):
 
 # the resident form with the field in shared memory: one CTA a sample (n = 128), clusters of four
 # (n = 256; 40 samples are more than one round of clusters), where AUTO takes it
-@pytest.mark.parametrize("n,R,ns", [(128, 6, 3), (128, 8, 155), (256, 4, 5), (256, 6, 40), (256, 8, 40)])
+@pytest.mark.parametrize("n,R,ns", [(128, 5, 3), (128, 6, 3), (128, 8, 155), (256, 4, 5), (256, 6, 40), (256, 8, 40)])
 @pytest.mark.parametrize("ic", [1, 2])
 def test_resident_clusters(gpu_lib, n, R, ns, ic):
     mf = gpu_lib
