@@ -321,8 +321,10 @@ def run_ours(args):
     peak_gbs, sm_max, peak_kind = load_peaks()
     # step kernels, then coefficients and the OoI finalisation, and either the padding kernel (tile
     # kernels) or the field reduction (row-streaming kernel, whose initial copy is a memcpy)
-    launches_per_solve = NSTEPS + 3
-    kernel_ms = ms_step / NSTEPS  # average step-kernel launch (upper bound: includes launch gaps)
+    # (the resident form: the coefficients and one launch for the whole solve)
+    on_chip = algo.startswith("resident")
+    launches_per_solve = 2 if on_chip else NSTEPS + 3
+    kernel_ms = ms_step / NSTEPS  # one time step (upper bound: includes launch gaps)
     bytes_launch = 8.0 * ns * N_LATTICE * N_LATTICE
     achieved = bytes_launch / (kernel_ms * 1e-3) / 1e9
     traffic = None
@@ -339,6 +341,16 @@ def run_ours(args):
     alu_peak = 152 * 128 * sm_max * 1e6 / 1e12
     alu_achieved = instr_per_pt * ns * N_LATTICE * N_LATTICE / (kernel_ms * 1e-3) / 1e12
 
+    kernel = ("resident_cluster_kernel" if on_chip else "step_rows_kernel" if algo.startswith("row-stream") else
+              "step_tma_kernel" if algo.startswith("prefix-tma") else "step_tile_kernel") + f" ({algo})"
+    roof_hbm = {"bound": "hbm", "achieved": achieved, "peak": peak_gbs, "unit": "GB/s", "frac": achieved / peak_gbs,
+                "traffic": traffic, "peak_kind": peak_kind, "kernel": kernel,
+                "algorithmic_bytes_per_launch": bytes_launch, "avg_launch_ms": kernel_ms}
+    # (on chip there is no field traffic between steps: the throughput in units of the prefix form)
+    roof_alu = {"bound": "alu", "achieved": alu_achieved, "peak": alu_peak, "unit": "T instr/s",
+                "frac": alu_achieved / alu_peak, "instr_per_point": instr_per_pt, "kernel": kernel,
+                "avg_time_step_ms": kernel_ms}
+
     if rank == 0:
         line = {"metric": METRIC, "value": value, "unit": METRIC, "n_gpus": ws, "steps": args.steps,
                 "warmup": args.warmup, "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak",
@@ -347,14 +359,7 @@ def run_ours(args):
                 "plain_form": None if plain_sps is None else {
                     "samples_per_s": plain_sps, "speedup_batched_vs_plain": batched_sps / plain_sps,
                     "what": "one sample per launch, one launch per step, direct disc sum"},
-                "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak_gbs, "unit": "GB/s",
-                             "frac": achieved / peak_gbs, "traffic": traffic, "peak_kind": peak_kind,
-                             "kernel": ("step_rows_kernel" if algo.startswith("row-stream") else
-                                        "step_tma_kernel" if algo.startswith("prefix-tma") else "step_tile_kernel")
-                                       + f" ({algo})", "algorithmic_bytes_per_launch": bytes_launch,
-                             "avg_launch_ms": kernel_ms},
-                "roofline_alu": {"bound": "alu", "achieved": alu_achieved, "peak": alu_peak, "unit": "T instr/s",
-                                 "frac": alu_achieved / alu_peak, "instr_per_point": instr_per_pt},
+                "roofline": roof_alu if on_chip else roof_hbm, "roofline_alu": roof_alu,
                 "e2e": None if e2e_s is None else {
                     "value": ws * ns * N_LATTICE * N_LATTICE * NSTEPS / e2e_s, "unit": METRIC,
                     "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,

@@ -75,7 +75,8 @@ typedef enum {
     MFMC_ALGO_DIRECT = 1,      /* sum over every disc point                       */
     MFMC_ALGO_PREFIX = 2,      /* in-register row prefix sums: O(R) adds per point */
     MFMC_ALGO_PREFIX_KAHAN = 3,/* prefix form with compensated accumulation       */
-    MFMC_ALGO_RESIDENT = 4,    /* whole field held in shared memory for all steps */
+    MFMC_ALGO_RESIDENT = 4,    /* whole field held on chip for all steps (AUTO and the
+                                  server also run n = 256 this way, in clusters of CTAs) */
     MFMC_ALGO_PLAIN = 5,       /* reference form: one sample per launch, direct   */
     MFMC_ALGO_PREFIX_TMA = 6,  /* prefix form, persistent CTAs, TMA double-buffered
                                   tiles of a ghost-framed field                   */
@@ -109,10 +110,10 @@ typedef enum {
                                   kernels: per step a column pass (FFT over y, product with the
                                   real transform of the disc weights, inverse) and a row pass
                                   (inverse row FFT, update, forward row FFT of the new rows);
-                                  n = 1024 in two launches per step; n = 64 and 128 in one
-                                  launch for the whole solve with the fields in shared memory
-                                  (register transforms); any other even n <= 128 whose odd part
-                                  is a product of 3, 5, 7 and 11 (the paper's h = 1/88) the same
+                                  n = 1024 in two launches per step; n = 64, 88 and 128 in
+                                  one launch for the whole solve with the fields in registers
+                                  (half-lattice transforms); any other even n <= 128 whose odd part
+                                  is a product of 3, 5, 7 and 11 the same
                                   way with mixed-radix transforms; cost independent of the
                                   horizon; any kernel and radius, periodic boundary,
                                   beta2 = 0; AUTO considers it */
@@ -333,9 +334,9 @@ mfmc_status mfmc_solve_batch(mfmc_model *const *models, const mfmc_sample_params
  * beta2 = 0, an even n <= 128 whose odd part is a product of 3, 5, 7 and 11, and any kernel and
  * horizon (the paper's nine models of Section 4 / Table 1, delta/h = 16.5 included), ONE
  * launch runs every sample's whole solve: persistent CTAs take (model, sample group) items,
- * heaviest model first, through an atomic ticket counter, and keep the fields in shared memory
- * for all steps, each item on the form MFMC_ALGO_SPECTRAL uses for its lattice (register
- * transforms on n = 64, four samples an item, and n = 128; mixed-radix transforms otherwise).
+ * heaviest model first, through an atomic ticket counter, and keep the fields on chip
+ * for all steps, each item on the form MFMC_ALGO_SPECTRAL uses for its lattice (half-lattice
+ * transforms on n = 64, four samples an item, n = 88 and 128; mixed-radix transforms otherwise).
  * Results equal those of MFMC_ALGO_SPECTRAL's solves of the same samples.
  *
  * Same arguments and results as mfmc_solve_batch; every sample runs >= 1 step.  Other inputs

@@ -32,7 +32,9 @@
 // One CTA per sample runs every step of its solve (every step of one launch, except with the
 // cuFFT sums: one step per launch, the state staying in global scratch between launches); its
 // fine-level vectors live in global scratch, the coarse multigrid levels that fit in shared
-// memory, and the CTA's reductions use a fixed order.  No CTA waits on another.  Every loop is
+// memory, and the CTA's reductions use a fixed order.  No CTA waits on another.  n = 64, 88 and
+// 128 (the paper's lattices) take the kernel of active_set_tile.cu, which holds the correction solve
+// on chip.  Every loop is
 // bounded; a Newton iteration that does not converge within its bound sets the status flag (a CG
 // solve that reaches its bound hands its iterate to the next Newton iteration).
 #include <cuda_runtime.h>
@@ -346,7 +348,7 @@ __global__ void __launch_bounds__(AS_NT) active_set_kernel(ActiveSetArgs a) {
         else if (a.own_fft) {  // (the coarse levels in shared memory hold nothing between steps)
             auto ld = [&](int y, int x) { return U[y * n + x]; };
             auto put = [&](int y, int x, double S) { G[y * n + x] = e2a * S + a.cF * U[y * n + x]; };
-            cta_disc_sums<0, double>(a.plan, as_smem, a.khat, a.tw, ld, put);
+            cta_disc_sums<double>(a.plan, as_smem, a.khat, a.tw, ld, put);
         } else as_for(n, [&](int y, int x, int i) {
             double S = 0.0;
             for (int dy = -R; dy <= R; ++dy) {

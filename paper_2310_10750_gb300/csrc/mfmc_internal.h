@@ -215,15 +215,15 @@ bool rows_batch_short(const Model &m, size_t ns);
 // The TMA pipeline with an explicit tile-shape variant (autotuner).
 mfmc_status run_solve_tma(Model &m, int kahan, int variant, const StepCoef *coef, const float *u0, size_t ns,
                           int nsteps, float *uT, double *ubar, double *ooi, cudaStream_t st);
-// The own-FFT spectral path (periodic, beta2 = 0): n = 1024 streamed, n = 64 and 128 resident in
-// the register-transform form, other even n <= 128 in the resident mixed-radix form.
+// The own-FFT spectral path (periodic, beta2 = 0): n = 1024 streamed, n = 64, 88 and 128 resident in
+// the tile form, other even n <= 128 in the resident mixed-radix form.
 bool spectral_supported(const Model &m);
 mfmc_status run_solve_spectral(Model &m, const StepCoef *coef, const float *u0, size_t ns, int nsteps, float *uT,
                                double *ubar, double *ooi, cudaStream_t st);
 // K^(ky, kx) / n^2 of the model's FP32 disc weights (summed in FP64), at [kx][ky].
 std::vector<float> spectral_khat(const Model &m, int n);
 // Resident spectral solves (spectral_resident.cu): one launch over the (model, sample group) items
-// of up to kSrMaxModels models with n <= 128 (register transforms on 64 and 128, mixed-radix
+// of up to kSrMaxModels models with n <= 128 (the tile form on 64, 88 and 128, mixed-radix
 // transforms on other n).
 constexpr int kSrMaxModels = 16;
 struct SrBatch {

@@ -18,7 +18,7 @@
 // transforms one sequence at a time in two buffers of n complex values of its own.  The 1-D
 // transform is a mixed-radix Stockham FFT (self-sorting, natural order in and out) with radices
 // 4, 2 and the odd primes up to 11, so it serves every even n whose odd part factors into those
-// primes (the paper's meshes 64, 88 = 8 x 11 and 128 among them).  Stage s with radix p after
+// primes (64, 88 and 128 have their own form, half_fft.cuh).  Stage s with radix p after
 // L = p_1 ... p_{s-1} (r = n / (L p)) maps the partial transforms y[k0][m] of length L of the
 // r p interleaved subsequences to those of length L p of r subsequences:
 //     y'[k0 + L k1][m] = sum_q W_p^(q k1) W_{Lp}^(q k0) y[k0][m + q r],
@@ -174,56 +174,6 @@ __device__ __noinline__ C *warp_fft(C *a, C *b, const FftPlan &P, const C *tw, i
     return a;
 }
 
-// The same transform with the plan fixed at compile time (the paper's meshes 64, 88 and 128):
-// every stage's radix, stride and butterfly count are constants, so the index arithmetic folds
-// and the radix dispatch disappears.
-struct CtPlan {
-    int stages = 0;
-    int radix[kFftMaxStages] = {};
-};
-__host__ __device__ constexpr CtPlan ct_plan(int n) {
-    CtPlan p{};
-    int m = n;
-    const int rs[6] = {11, 7, 5, 3, 4, 2};
-    for (int i = 0; i < 6; ++i)
-        while (m % rs[i] == 0 && p.stages < kFftMaxStages) {
-            p.radix[p.stages++] = rs[i];
-            m /= rs[i];
-        }
-    return p;
-}
-
-template <int N, int S, int L, bool INV, typename C>
-__device__ __forceinline__ C *ct_fft_stages(C *a, C *b, const C *tw, int lane) {
-    constexpr CtPlan P = ct_plan(N);
-    if constexpr (S == P.stages) {
-        return a;
-    } else {
-        constexpr int p = P.radix[S], r = N / (L * p), nb = N / p;
-#pragma unroll
-        for (int b0 = 0; b0 < nb; b0 += 32) {
-            const int bi = b0 + lane;
-            if (nb % 32 == 0 || bi < nb) {
-                const int k0 = bi / r, m = bi - k0 * r;
-                fft_butterfly<p, INV>(a + k0 * r * p + m, b + k0 * r + m, r, L * r, k0 * r, tw, N);
-            }
-        }
-        __syncwarp();
-        return ct_fft_stages<N, S + 1, L * p, INV>(b, a, tw, lane);
-    }
-}
-
-// n-point transform by one warp; N > 0: the compile-time plan of N (n == N), else P's.
-template <int N, bool INV, typename C>
-__device__ __forceinline__ C *warp_fft_any(C *a, C *b, const FftPlan &P, const C *tw, int lane) {
-    if constexpr (N > 0) {
-        static_assert(ct_plan(N).stages > 0, "no plan");
-        return ct_fft_stages<N, 0, 1, INV>(a, b, tw, lane);
-    } else {
-        return warp_fft<INV>(a, b, P, tw, lane);
-    }
-}
-
 // Shared memory of cta_disc_sums for an n x n lattice and `warps` warps: the half spectrum,
 // then two buffers of n complex values per warp.
 template <typename T>
@@ -235,12 +185,12 @@ __host__ __device__ constexpr size_t fft_smem_bytes(int n, int warps) {
 // u; st(y, x, S) receives each sum once (rows in pairs, any order).  smem: fft_smem_bytes(n,
 // warps of the CTA) bytes, 16-byte aligned; khat: K^(ky, kx) / n^2 at [ky][n/2 + 1] (global);
 // tw: W_n^j, j < n (global).  Begins and ends with a CTA barrier, so smem may be shared with
-// other phases of the caller.  N > 0: n == N, transformed with the compile-time plan.
-template <int N, typename T, typename Ld, typename St>
+// other phases of the caller.
+template <typename T, typename Ld, typename St>
 __device__ __noinline__ void cta_disc_sums(const FftPlan &P, void *smem, const T *khat,
                                            const typename FftCx<T>::t *tw, Ld ld, St st) {
     using C = typename FftCx<T>::t;
-    const int n = N > 0 ? N : P.n, NH = n / 2 + 1, nw = blockDim.x >> 5, w = threadIdx.x >> 5,
+    const int n = P.n, NH = n / 2 + 1, nw = blockDim.x >> 5, w = threadIdx.x >> 5,
               lane = threadIdx.x & 31;
     C *spec = reinterpret_cast<C *>(smem);
     C *A = spec + (size_t)n * NH + (size_t)w * 2 * n, *B = A + n;
@@ -249,7 +199,7 @@ __device__ __noinline__ void cta_disc_sums(const FftPlan &P, void *smem, const T
     for (int pr = w; pr < n / 2; pr += nw) {  // forward row pass
         for (int x = lane; x < n; x += 32) A[x] = fcx<C>(ld(2 * pr, x), ld(2 * pr + 1, x));
         __syncwarp();
-        const C *Z = warp_fft_any<N, false>(A, B, P, tw, lane);
+        const C *Z = warp_fft<false>(A, B, P, tw, lane);
         C *sa = spec + (size_t)(2 * pr) * NH, *sb = sa + NH;
         for (int k = lane; k <= n / 2; k += 32) {
             const C zk = Z[k], zm = Z[k == 0 ? 0 : n - k];
@@ -262,13 +212,13 @@ __device__ __noinline__ void cta_disc_sums(const FftPlan &P, void *smem, const T
     for (int c = w; c < NH; c += nw) {  // column pass
         for (int ky = lane; ky < n; ky += 32) A[ky] = spec[(size_t)ky * NH + c];
         __syncwarp();
-        C *Y = warp_fft_any<N, false>(A, B, P, tw, lane);
+        C *Y = warp_fft<false>(A, B, P, tw, lane);
         for (int ky = lane; ky < n; ky += 32) {
             const T k = khat[(size_t)ky * NH + c];
             Y[ky] = fcx<C>(Y[ky].x * k, Y[ky].y * k);
         }
         __syncwarp();
-        const C *X = warp_fft_any<N, true>(Y, Y == A ? B : A, P, tw, lane);
+        const C *X = warp_fft<true>(Y, Y == A ? B : A, P, tw, lane);
         for (int ky = lane; ky < n; ky += 32) spec[(size_t)ky * NH + c] = X[ky];
         __syncwarp();
     }
@@ -285,7 +235,7 @@ __device__ __noinline__ void cta_disc_sums(const FftPlan &P, void *smem, const T
             }
         }
         __syncwarp();
-        const C *S = warp_fft_any<N, true>(A, B, P, tw, lane);
+        const C *S = warp_fft<true>(A, B, P, tw, lane);
         for (int x = lane; x < n; x += 32) {
             const C s = S[x];
             st(2 * pr, x, s.x);

@@ -372,7 +372,7 @@ __device__ __noinline__ void sq_solve_generic(const SqModelDev &M, int s, float 
     const StepCoef cf = M.coef[s];
     const int steps = M.steps_ps ? M.steps_ps[s] : M.nsteps;
     for (int k = 0; k < steps; ++k)
-        cta_disc_sums<0, float>(
+        cta_disc_sums<float>(
             M.plan, fsm, M.khat, M.tw, [&](int y, int x) { return u[y * n + x]; },
             [&](int y, int x, float S) {
                 const float uv = u[y * n + x];
