@@ -256,12 +256,11 @@ mfmc_status run_solve_active_set(Model &m, const double *eps_dev, const float *u
                                  float *uT, double *ubar, double *ooi, cudaStream_t st);
 // Whether an algorithm can run this model.
 bool algo_supported(const Model &m, int algo);
-// Whether a caller may name it for this model: the row kernel's R = 12 and 16 and the resident
-// form's n = 256 are AUTO's (and the server's) choice only.
-inline bool algo_selectable(const Model &m, int algo) {
-    return algo_supported(m, algo) && !(algo == MFMC_ALGO_ROWS && m.R > 8) &&
-           !(algo == MFMC_ALGO_RESIDENT && m.d.n > 128);
-}
+// Whether a caller may name it for this model.  The row kernel's R = 12 and 16 and the resident form's
+// n = 256 are AUTO's (and the server's) choice: a caller may name them once AUTO has chosen them for
+// the lattice and horizon in this process, so that the algorithm mfmc_model_query reports can be
+// asked for.
+bool algo_selectable(const Model &m, int algo);
 // Autotuner: time the candidate algorithms on this model once and cache the winner.
 mfmc_status autotune(Model &m, cudaStream_t st);
 

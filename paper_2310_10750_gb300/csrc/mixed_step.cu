@@ -284,7 +284,7 @@ extern "C" mfmc_status mfmc_solve_batch_mixed(mfmc_model *const *models, const m
     for (int g = 0; g < ng; ++g) {
         mfmc_model *m = order[g];
         const auto &idx = groups[m];
-        resident[g] = spec_route || algo_selectable(*m, MFMC_ALGO_RESIDENT) ? 1 : 0;
+        resident[g] = spec_route || (m->d.n <= 128 && algo_supported(*m, MFMC_ALGO_RESIDENT)) ? 1 : 0;
         if (!resident[g]) queue.push_back(g);
         mfmc_status s = ensure_group(W.g[g], *m, idx.size(), !resident[g], st, &W.generation);
         if (s != MFMC_OK) return s;

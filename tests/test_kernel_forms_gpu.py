@@ -118,16 +118,28 @@ def test_rows_and_tiles_agree_on_each_side_of_the_batch_rule(gpu_lib, n, R, many
 
 
 def test_forms_auto_alone_chooses_stay_refused(gpu_lib):
+    # lattices that AUTO has not tuned in this process
     import torch
     mf = gpu_lib
-    u0 = torch.zeros((1, 512, 512), dtype=torch.float32, device="cuda")
-    for n, R, algo in ((512, 16, mf.ALGO_ROWS), (256, 12, mf.ALGO_ROWS), (256, 8, mf.ALGO_RESIDENT)):
+    u0 = torch.zeros((1, 768, 768), dtype=torch.float32, device="cuda")
+    for n, R in ((640, 16), (768, 12)):
         with pytest.raises(mf.MfmcError) as e:
-            mf.Model(n=n, delta=R / n, algo=algo)
+            mf.Model(n=n, delta=R / n, algo=mf.ALGO_ROWS)
         assert e.value.status == mf.MFMC_EINVAL
         with pytest.raises(mf.MfmcError) as e:
-            mf.mfmc_solve_fields_algo(mf.Model(n=n, delta=R / n, nsteps=1), algo, u0, 1)
+            mf.mfmc_solve_fields_algo(mf.Model(n=n, delta=R / n, nsteps=1), mf.ALGO_ROWS, u0, 1)
         assert e.value.status == mf.MFMC_EINVAL
+
+
+@pytest.mark.parametrize("n,R,ns", [(256, 8, 5), (512, 16, 45)])
+def test_the_algorithm_a_query_reports_can_be_asked_for(gpu_lib, n, R, ns):
+    mf = gpu_lib
+    kw = dict(n=n, delta=R / n, eps=0.02, tau=1e-3, ic=2, nsteps=2)
+    ga = mf.Model(**kw)
+    _, ua, fa = fields(mf, ga, seeds_of(ns, 31), [0, ns - 1])
+    gb = mf.Model(algo=ga.info().algo, **kw)
+    _, ub, fb = fields(mf, gb, seeds_of(ns, 31), [0, ns - 1])
+    assert np.array_equal(ua, ub) and np.array_equal(fa, fb)
 
 
 @pytest.mark.parametrize("n", [64, 88, 128])
