@@ -279,21 +279,26 @@ std::vector<double> khat64_host(const Model &m, int n) {
         const int w = m.widths[ady];
         for (int kx = 0; kx < nh1; ++kx) {
             double c = 0.0;
+            int j = (int)((long long)kx * (n - w) % n);  // kx dx mod n, stepped
             for (int dx = -w; dx <= w; ++dx) {
                 const double wt = m.d.kernel == MFMC_KERNEL_CONSTANT ? 1.0 : m.wtab64[dx * dx + ady * ady];
-                c += wt * cs[(size_t)(((long)kx * dx) % n + n) % n];
+                c += wt * cs[j];
+                j += kx;
+                if (j >= n) j -= n;
             }
             C[(size_t)ady * nh1 + kx] = c;
         }
     }
     const double inv_nn = 1.0 / ((double)n * n);
-    for (int ky = 0; ky < n; ++ky)
-        for (int kx = 0; kx < nh1; ++kx) {
-            double k = 0.0;
-            for (int dy = -m.R; dy <= m.R; ++dy)
-                k += C[(size_t)(dy < 0 ? -dy : dy) * nh1 + kx] * cs[(size_t)(((long)ky * dy) % n + n) % n];
-            K[(size_t)ky * nh1 + kx] = k * inv_nn;
+    for (int ky = 0; ky < n; ++ky) {
+        double *row = &K[(size_t)ky * nh1];
+        for (int dy = -m.R; dy <= m.R; ++dy) {
+            const double c = cs[(size_t)(((long)ky * dy) % n + n) % n];
+            const double *a = &C[(size_t)(dy < 0 ? -dy : dy) * nh1];
+            for (int kx = 0; kx < nh1; ++kx) row[kx] += a[kx] * c;
         }
+        for (int kx = 0; kx < nh1; ++kx) row[kx] *= inv_nn;
+    }
     return K;
 }
 

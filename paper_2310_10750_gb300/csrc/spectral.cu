@@ -500,27 +500,34 @@ static std::vector<double> spectral_khat64(const Model &m, int n) {
     const int R = m.R, half = n / 2 + 1;
     std::vector<double> cs(n);
     for (int i = 0; i < n; ++i) cs[i] = std::cos(2.0 * M_PI * (double)i / (double)n);
-    // A[dy][kx] = sum_dx w(dx, dy) cos(2 pi kx dx / n), dy = 0..R
+    // A[dy][kx] = sum_dx w(dx, dy) cos(2 pi kx dx / n), dy = 0..R (the index of the cosine table
+    // stepped: a remainder per term took most of a new model's first solve)
     std::vector<double> A((size_t)(R + 1) * half, 0.0);
     for (int dy = 0; dy <= R; ++dy) {
         const int wd = m.widths[dy];
         for (int kx = 0; kx < half; ++kx) {
             double s = 0.0;
+            int j = (int)((long long)kx * (n - wd) % n);
             for (int dx = -wd; dx <= wd; ++dx) {
                 const double wt = m.d.kernel == MFMC_KERNEL_CONSTANT ? 1.0 : (double)m.wtab[dx * dx + dy * dy];
-                s += wt * cs[(size_t)(((long long)kx * (dx + n)) % n)];
+                s += wt * cs[j];
+                j += kx;
+                if (j >= n) j -= n;
             }
             A[(size_t)dy * half + kx] = s;
         }
     }
-    std::vector<double> kh((size_t)half * n);
+    std::vector<double> kh((size_t)half * n), row(half);
     const double scale = 1.0 / ((double)n * n);
-    for (int ky = 0; ky < n; ++ky)
-        for (int kx = 0; kx < half; ++kx) {
-            double s = A[kx];  // dy = 0
-            for (int dy = 1; dy <= R; ++dy) s += 2.0 * cs[(size_t)((long long)ky * dy % n)] * A[(size_t)dy * half + kx];
-            kh[(size_t)kx * n + ky] = s * scale;
+    for (int ky = 0; ky < n; ++ky) {
+        for (int kx = 0; kx < half; ++kx) row[kx] = A[kx];  // dy = 0
+        for (int dy = 1; dy <= R; ++dy) {
+            const double c = 2.0 * cs[(size_t)((long long)ky * dy % n)];
+            const double *a = &A[(size_t)dy * half];
+            for (int kx = 0; kx < half; ++kx) row[kx] += c * a[kx];
         }
+        for (int kx = 0; kx < half; ++kx) kh[(size_t)kx * n + ky] = row[kx] * scale;
+    }
     return kh;
 }
 
