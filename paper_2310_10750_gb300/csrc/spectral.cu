@@ -696,6 +696,7 @@ mfmc_status run_solve_spectral(Model &m, const StepCoef *coef, const float *u0, 
     if (m.d.n == 64) return run_solve_spectral_tile<64, 4>(m, coef, u0, ns, nsteps, uT, ubar, ooi, st);
     if (m.d.n != kN) return run_solve_spectral_resident(m, coef, u0, ns, nsteps, uT, ubar, ooi, st);
     mfmc_status s = spectral_prepare(m, ns);
+    if (s == MFMC_OK) s = grow_buffer(&m.partials, &m.partials_cap, ns * kOoiChunks);
     if (s != MFMC_OK) return s;
     SpectralState &f = *m.spectral;
     int dev = 0, sms = 0;
@@ -729,8 +730,6 @@ mfmc_status run_solve_spectral(Model &m, const StepCoef *coef, const float *u0, 
         MFMC_LAUNCHED("spectral launch 3");
         src = dst;
     }
-    s = grow_buffer(&m.partials, &m.partials_cap, ns * kOoiChunks);
-    if (s != MFMC_OK) return s;
     return launch_field_ooi_chunks(src, ns, kN, m.partials, kOoiChunks, ubar, ooi, st);
 }
 
