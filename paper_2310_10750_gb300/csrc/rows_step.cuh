@@ -25,9 +25,10 @@
 // add itself, acc[k] = acc[k + 1] + h, so the row loop is one short body.  (A ring of 2R + 1 static
 // slots, unrolled by its period, is as fast at R = 8, 58.2 against 57.9 us a step of 512 samples of
 // 256^2, but at R = 16 its 33 rows of code miss the instruction cache: 1.92 us a sample-step of
-// 512^2 against 0.84, the tile kernel 1.14.)  After staged row q the output row q - 2R is complete and is finished at once (update, projection, store).  The OoI is
-// reduced afterwards from the final fields (rows_ooi_kernel), so it does not depend on how the
-// rows were split.
+// 512^2 against 0.84, the tile kernel 1.14.  Two CTAs of half as many warps an SM: 512^2, R = 16 58.0
+// -> 58.7 us a step of 64 samples, R = 8 34.3 -> 39.3.)  After staged row q the output row q - 2R is
+// complete and is finished at once (update, projection, store).  The OoI is reduced afterwards from
+// the final fields (rows_ooi_kernel), so it does not depend on how the rows were split.
 //
 // Consecutive steps are launched as programmatic dependents: a step's CTAs set up their
 // barriers and walk while the previous step drains, and wait for its completion
