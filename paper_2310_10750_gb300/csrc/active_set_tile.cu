@@ -24,6 +24,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cfloat>
 
 #include "active_set_tile.cuh"
 #include "spectral_tile.cuh"
@@ -152,15 +153,17 @@ struct At {
         rpar ^= 1;
         return t;
     }
-    // CTA-wide maximum of non-negative values (their bit patterns order as unsigned integers).
-    __device__ __forceinline__ float max(float v) {
-        const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(v));
+    // CTA-wide maximum of unsigned integers.
+    __device__ __forceinline__ unsigned max_bits(unsigned v) {
+        const unsigned m = __reduce_max_sync(0xffffffffu, v);
         if (lane == 0) red[rpar * 32 + warp] = __uint_as_float(m);
         __syncthreads();
         const unsigned t = __reduce_max_sync(0xffffffffu, lane < K::NW ? __float_as_uint(red[rpar * 32 + lane]) : 0u);
         rpar ^= 1;
-        return __uint_as_float(t);
+        return t;
     }
+    // CTA-wide maximum of non-negative values (their bit patterns order as unsigned integers).
+    __device__ __forceinline__ float max(float v) { return __uint_as_float(max_bits(__float_as_uint(v))); }
 
     template <int L>
     __device__ __forceinline__ float tb2l() const { return tb2 * (1.0f / (1 << (2 * L))); }
@@ -572,7 +575,7 @@ __global__ void __launch_bounds__(AtCfg<N>::NT, MINB) active_set_tile_kernel(con
             ++n_newton;
             // FP64 residual F(w), the inactive set, and the right-hand side f = -F of J d = -F
             float f[RW][CW];
-            float fmax = 0.0f;
+            unsigned fhi = 0u;  // maximum of the high words of |F|: a NaN's lies above every number's
             unsigned now = 0u;
             {
                 double up[CW], cur[CW], dn[CW];
@@ -599,7 +602,7 @@ __global__ void __launch_bounds__(AtCfg<N>::NT, MINB) active_set_tile_kernel(con
                         const double F = fma(wdiag, cur[c], fma(-tb2h, S, xc - u[c]));
                         now |= in ? 1u << (y * CW + c) : 0u;
                         f[y][c] = act ? -(float)F : 0.0f;
-                        fmax = fmaxf(fmax, fabsf(f[y][c]));
+                        fhi = umax(fhi, (unsigned)__double2hiint(F) & 0x7fffffffu);
                     }
 #pragma unroll
                     for (int c = 0; c < CW; ++c) {
@@ -610,13 +613,17 @@ __global__ void __launch_bounds__(AtCfg<N>::NT, MINB) active_set_tile_kernel(con
             }
             const bool changed = __syncthreads_or(act && now != t.mask);
             t.mask = now;
-            fmax = t.max(fmax);
-            if (it > 1 && !changed && fmax <= 1e-11f) break;
-            if (it > a.newton_max) {
+            // the largest |F| with that high word: what passes meets the bound in full
+            const double fbound = __hiloint2double((int)t.max_bits(act ? fhi : 0u), -1);
+            if (it > 1 && !changed && fbound <= 1e-11) break;
+            // the bound on the passes, or a residual that no pass mends (a NaN or an infinity, which the
+            // correction would carry to every point): the sample's solve stops
+            if (it > a.newton_max || !(fbound < INFINITY)) {
                 failed = true;
                 break;
             }
-            if (fmax == 0.0f) continue;  // F = 0 with a new active set: the next pass confirms it
+            const float fmax = (float)fbound;
+            if (fmax < FLT_MIN) continue;  // F = 0 with a new active set: the next pass confirms it
             at_tail_diagonals<N>(t);
             const float sc = 1.0f / fmax;  // scaled to max |f| = 1
 #pragma unroll

@@ -1,0 +1,57 @@
+"""The beta2 > 0 solver's on-chip kernel (n = 64, 88, 128): what it reports when a solve cannot
+succeed.  n = 32 runs the other kernel, whose report is the one to match."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def model(mf, n, R, **kw):
+    return mf.Model(n=n, delta=R / n, eps=0.04219, tau=0.01, nsteps=3, ic=2, beta2=0.05, **kw)
+
+
+# discs of 49 points (the direct sum, which leaves a NaN where it is) and of 197 (the transforms,
+# which spread it)
+@pytest.mark.parametrize("n", [32, 64, 88, 128])
+@pytest.mark.parametrize("R", [4, 8])
+def test_non_finite_samples_report_timeout(gpu_lib, n, R):
+    mf = gpu_lib
+    g = model(mf, n, R)
+    seeds = np.arange(3, dtype=np.uint64) + 17
+    good, _ = mf.mfmc_solve_batch([g] * 3, seeds)
+    mu, eta = [0.95] * 4, [[0.0, 0.0]] * 4
+    bad = [mf.make_params(3, theta=[None, ([np.nan] + mu[1:], eta), None]),
+           mf.make_params(3, theta=[None, (mu, [[np.inf, 0.0]] + eta[1:]), None]),
+           mf.make_params(3, eps=[0.04219, np.inf, 0.04219])]
+    for p in bad:
+        with pytest.raises(mf.MfmcError) as e:
+            mf.mfmc_solve_batch([g] * 3, seeds, params=p)
+        assert e.value.status == mf.MFMC_ETIMEOUT
+        again, _ = mf.mfmc_solve_batch([g] * 3, seeds)  # the model and the device stay usable
+        assert np.array_equal(again, good)
+
+
+@pytest.mark.parametrize("n", [64, 88, 128])
+@pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf])
+def test_one_non_finite_value_stops_its_sample_alone(gpu_lib, n, value):
+    # a stopped sample's outputs are left as they were; its neighbours keep every bit
+    import torch
+    mf = gpu_lib
+    g = model(mf, n, 8)
+    u0 = torch.empty((3, n, n), dtype=torch.float32, device="cuda")
+    mf.mfmc_init_fields(g, np.arange(3, dtype=np.uint64) + 5, u0)
+
+    def solve(u):
+        uT = torch.full_like(u, 7.0)
+        ooi = torch.full((3,), 7.0, dtype=torch.float64, device="cuda")
+        mf.mfmc_solve_fields(g, u, 3, uT=uT, ooi=ooi)
+        torch.cuda.synchronize()
+        return uT.cpu().numpy(), ooi.cpu().numpy()
+
+    uT, ooi = solve(u0)
+    v0 = u0.clone()
+    v0[1, n // 2, 3] = value
+    vT, voi = solve(v0)
+    assert np.all(vT[1] == 7.0) and voi[1] == 7.0
+    for i in (0, 2):
+        assert np.array_equal(vT[i], uT[i]) and voi[i] == ooi[i]
