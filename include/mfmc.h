@@ -275,6 +275,8 @@ mfmc_status mfmc_init_fields(const mfmc_model *model, const mfmc_sample_params *
  *   uT    device, [ns][n][n] FP32 final fields, or NULL
  *   ubar  device, ns FP64 spatial means of u(T), or NULL
  *   ooi   device, ns FP64 outputs of interest, or NULL
+ * Each pointer needs the alignment of its type (u0 and uT: 4 bytes, else MFMC_EINVAL).  Fields that
+ * start on a 16-byte boundary are used in place; others may pass through the library's scratch.
  * Scratch (two field buffers for the streaming kernels) is owned by the library and
  * reused across calls.  ns == 0 is a no-op. */
 mfmc_status mfmc_solve_fields(const mfmc_model *model, const double *eps, const float *u0,
@@ -297,7 +299,8 @@ mfmc_status mfmc_solve_fields_algo(const mfmc_model *model, int algo, const doub
  * exit.  Limits: ns <= 4096, ns * n * n * 4 <= 16,482,304 bytes (e.g. 62 fields of
  * 256 x 256, 1006 fields of 64 x 64), ns * tiles <= 65536; larger batches return
  * MFMC_EINVAL with the limits in the message.  Constant kernel and R in
- * {1,2,3,4,5,6,8,11,12,16,22,24,32} only.  The first call on a device looks up the
+ * {1,2,3,4,5,6,8,11,12,16,22,24,32} only; u0 and uT on 16-byte boundaries, else MFMC_EINVAL.  The
+ * first call on a device looks up the
  * array's device address (cudaGetSymbolAddress) and keeps it for the life of the process,
  * so make it before any stream capture, and do not use this call after cudaDeviceReset on
  * that device (the kept address would then be stale).  All calls share the one array and

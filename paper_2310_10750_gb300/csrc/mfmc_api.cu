@@ -49,6 +49,8 @@ Model::~Model() {
     cudaFree(theta_tmp);
     cudaFree(u0buf);
     cudaFree(resbuf);
+    cudaFree(u0_copy);
+    cudaFree(uT_copy);
     cudaFree(padA);
     cudaFree(padB);
     cudaFree(d_status);
@@ -319,24 +321,9 @@ mfmc_status mfmc_init_fields(const mfmc_model *cm, const mfmc_sample_params *par
     return MFMC_OK;
 }
 
-static mfmc_status solve_impl(mfmc_model *m, int algo, const double *eps, const float *u0, size_t ns, float *uT,
-                              double *ubar, double *ooi, cudaStream_t st, int nsteps = -1) {
-    if (nsteps < 0) nsteps = m->d.nsteps;
-    if (ns == 0) return MFMC_OK;
-    if (!u0) return fail(MFMC_EINVAL, "NULL u0");
-    if (uT && uT == u0) return fail(MFMC_EINVAL, "uT must not alias u0");
-    if (ns > (size_t)kMaxNs) return fail(MFMC_EINVAL, "too many samples");
-    std::lock_guard<std::mutex> lk(m->mu);
-    if (algo == MFMC_ALGO_AUTO) {
-        if (!m->tuned) {
-            mfmc_status s = autotune(*m, st);
-            if (s != MFMC_OK) return s;
-        }
-        algo = m->algo;
-        if (algo == MFMC_ALGO_ROWS && rows_batch_short(*m, ns)) algo = MFMC_ALGO_PREFIX_TMA;
-    } else if (!algo_selectable(*m, algo)) {
-        return fail(MFMC_EINVAL, "algorithm %d does not support this model", algo);
-    }
+// The solve by one algorithm, the model's lock held, u0 and uT aligned as its kernels need.
+static mfmc_status solve_by(mfmc_model *m, int algo, const double *eps, const float *u0, size_t ns, float *uT,
+                            double *ubar, double *ooi, cudaStream_t st, int nsteps) {
     if (algo == MFMC_ALGO_ACTIVE_SET) return run_solve_active_set(*m, eps, u0, ns, nsteps, uT, ubar, ooi, st);
     mfmc_status s = grow(&m->coef, &m->coef_cap, ns);
     if (s != MFMC_OK) return s;
@@ -390,6 +377,47 @@ static mfmc_status solve_impl(mfmc_model *m, int algo, const double *eps, const 
     }
     m->gkey = key();
     return MFMC_OK;
+}
+
+static bool aligned_to(const void *p, size_t bytes) { return (uintptr_t)p % bytes == 0; }
+
+static mfmc_status solve_impl(mfmc_model *m, int algo, const double *eps, const float *u0, size_t ns, float *uT,
+                              double *ubar, double *ooi, cudaStream_t st, int nsteps = -1) {
+    if (nsteps < 0) nsteps = m->d.nsteps;
+    if (ns == 0) return MFMC_OK;
+    if (!u0) return fail(MFMC_EINVAL, "NULL u0");
+    if (uT && uT == u0) return fail(MFMC_EINVAL, "uT must not alias u0");
+    if (!aligned_to(u0, sizeof(float)) || !aligned_to(uT, sizeof(float)))
+        return fail(MFMC_EINVAL, "u0 and uT must be aligned as floats");
+    if (ns > (size_t)kMaxNs) return fail(MFMC_EINVAL, "too many samples");
+    std::lock_guard<std::mutex> lk(m->mu);
+    if (algo == MFMC_ALGO_AUTO) {
+        if (!m->tuned) {
+            mfmc_status s = autotune(*m, st);
+            if (s != MFMC_OK) return s;
+        }
+        algo = m->algo;
+        if (algo == MFMC_ALGO_ROWS && rows_batch_short(*m, ns)) algo = MFMC_ALGO_PREFIX_TMA;
+    } else if (!algo_selectable(*m, algo)) {
+        return fail(MFMC_EINVAL, "algorithm %d does not support this model", algo);
+    }
+    const size_t nn = (size_t)m->d.n * m->d.n;
+    const bool copy_in = nsteps > 0 && !aligned_to(u0, 16) && wide_u0(*m, algo);
+    const bool copy_out = nsteps > 0 && !aligned_to(uT, 16) && wide_uT(*m, algo);
+    if (copy_in) {
+        mfmc_status s = grow_buffer(&m->u0_copy, &m->u0_copy_cap, ns * nn);
+        if (s != MFMC_OK) return s;
+        MFMC_CUDA(cudaMemcpyAsync(m->u0_copy, u0, ns * nn * sizeof(float), cudaMemcpyDeviceToDevice, st));
+        u0 = m->u0_copy;
+    }
+    if (copy_out) {
+        mfmc_status s = grow_buffer(&m->uT_copy, &m->uT_copy_cap, ns * nn);
+        if (s != MFMC_OK) return s;
+    }
+    mfmc_status s = solve_by(m, algo, eps, u0, ns, copy_out ? m->uT_copy : uT, ubar, ooi, st, nsteps);
+    if (s == MFMC_OK && copy_out)
+        MFMC_CUDA(cudaMemcpyAsync(uT, m->uT_copy, ns * nn * sizeof(float), cudaMemcpyDeviceToDevice, st));
+    return s;
 }
 
 mfmc_status mfmc_solve_fields(const mfmc_model *cm, const double *eps, const float *u0, size_t ns, float *uT,

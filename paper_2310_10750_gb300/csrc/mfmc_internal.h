@@ -81,6 +81,9 @@ struct Model {
     double *resbuf = nullptr;
     size_t res_cap = 0;
     cudaStream_t stream = nullptr;
+    // aligned copies of a caller's fields that do not start on a 16-byte boundary
+    float *u0_copy = nullptr, *uT_copy = nullptr;
+    size_t u0_copy_cap = 0, uT_copy_cap = 0;  // floats
     // ghost-framed scratch of the TMA path: [cap][P][P], P = n + 2 G, and its tensor maps
     float *padA = nullptr, *padB = nullptr;
     size_t pad_cap = 0;
@@ -254,6 +257,10 @@ mfmc_status fft64_disc_sums(Model &m, const double *u, size_t u_dist, double *S,
 // CG corrections, one CTA per sample); eps_dev: per-sample eps (FP64) or nullptr for the nominal eps.
 mfmc_status run_solve_active_set(Model &m, const double *eps_dev, const float *u0, size_t ns, int nsteps,
                                  float *uT, double *ubar, double *ooi, cudaStream_t st);
+// Whether an algorithm's kernels access the caller's initial (final) fields 16 bytes at a time.  solve_impl
+// passes such fields through aligned copies when they do not start on a 16-byte boundary.
+bool wide_u0(const Model &m, int algo);
+bool wide_uT(const Model &m, int algo);
 // Whether an algorithm can run this model.
 bool algo_supported(const Model &m, int algo);
 // Whether a caller may name it for this model.  The row kernel's R = 12 and 16 and the resident form's

@@ -15,6 +15,14 @@
 
 namespace mfmc {
 
+// Four floats of a field that need be aligned as floats only: one load when `wide` (the field starts on
+// a 16-byte boundary; rows are multiples of 16 bytes), else four.
+__device__ __forceinline__ bool wide_access(const void *field) { return (reinterpret_cast<uintptr_t>(field) & 15) == 0; }
+__device__ __forceinline__ float4 load4(const float *p, bool wide) {
+    if (wide) return __ldg(reinterpret_cast<const float4 *>(p));
+    return make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
+}
+
 // ----------------------------------------------------------------------------- ICs
 // Built in FP64 with explicitly rounded operations (no contraction) and rounded to FP32.
 __device__ double ic_normal(uint64_t seed, uint32_t q) {
@@ -378,10 +386,11 @@ mfmc_status launch_field_ooi(const float *u, size_t ns, int n, double *ubar, dou
 // FP64 adds run at two a clock an SM, so one CTA per field took 606 us on 64 fields of 1024^2.
 __global__ void __launch_bounds__(256) field_chunks_kernel(const float *u, int per, double *partials) {
     __shared__ double red[8];
-    const float4 *f = reinterpret_cast<const float4 *>(u + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * per);
+    const float *f = u + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * per;
+    const bool wide = wide_access(u);
     double t = 0.0;
     for (int i = threadIdx.x; i < per / 4; i += 256) {
-        const float4 v = f[i];
+        const float4 v = load4(f + 4 * i, wide);
         t += ((double)v.x + (double)v.y) + ((double)v.z + (double)v.w);
     }
     t = block_sum_fixed<256>(t, red);
@@ -437,13 +446,39 @@ bool algo_supported(const Model &m, int algo) {
     }
 }
 
+// Whether DIRECT or PREFIX runs this model on the register-tiled kernel (else the generic one).
+static bool tiled_form(const Model &m, int algo) {
+    const TileLauncher *L = tile_launcher(m.R);
+    return m.d.kernel == MFMC_KERNEL_CONSTANT && L && m.d.bc == MFMC_BC_PERIODIC && m.integer_R &&
+           ((algo == MFMC_ALGO_DIRECT && L->fn[0]) || (algo == MFMC_ALGO_PREFIX && L->fn[1]));
+}
+
+bool wide_u0(const Model &m, int algo) {
+    switch (algo) {
+        case MFMC_ALGO_ROWS:        // copied whole
+        case MFMC_ALGO_PREFIX_TMA:  // framed by pad_fields_kernel
+        case MFMC_ALGO_PREFIX_KAHAN:
+        case MFMC_ALGO_WEIGHTED:
+        case MFMC_ALGO_ACTIVE_SET: return false;
+        case MFMC_ALGO_SPECTRAL: return m.d.n > 128;
+        default: return true;
+    }
+}
+
+bool wide_uT(const Model &m, int algo) {
+    switch (algo) {
+        case MFMC_ALGO_SPECTRAL:
+        case MFMC_ALGO_ACTIVE_SET:
+        case MFMC_ALGO_PLAIN: return false;
+        case MFMC_ALGO_DIRECT: return tiled_form(m, algo);
+        default: return true;
+    }
+}
+
 static int tiles_for(const Model &m, int algo, int *tiles_x) {
     int tx = GEN_TX, ty = GEN_TY;
     const TileLauncher *L = tile_launcher(m.R);
-    const bool constant = m.d.kernel == MFMC_KERNEL_CONSTANT;
-    const bool tiled = constant && L && m.d.bc == MFMC_BC_PERIODIC && m.integer_R &&
-                       ((algo == MFMC_ALGO_DIRECT && L->fn[0]) || algo == MFMC_ALGO_PREFIX);
-    if (tiled) {
+    if (tiled_form(m, algo)) {
         tx = L->tx;
         ty = L->ty;
     }
@@ -471,6 +506,7 @@ static mfmc_status launch_generic(const Model &m, const GenericArgs &base, size_
 __global__ void pad_fields_kernel(const float *u, float *dst, int n, int G, size_t ns, int collar, float uI) {
     const int P = n + 2 * G, P4 = P / 4;
     const size_t total = ns * (size_t)P * P4;
+    const bool wide = wide_access(u);
     for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total;
          idx += (size_t)gridDim.x * blockDim.x) {
         const size_t smp = idx / ((size_t)P * P4);
@@ -481,7 +517,7 @@ __global__ void pad_fields_kernel(const float *u, float *dst, int n, int G, size
             v = make_float4(uI, uI, uI, uI);
         } else {
             const int y = wrap_idx(py - G, n), x = wrap_idx(px - G, n);
-            v = __ldg(reinterpret_cast<const float4 *>(u + smp * (size_t)n * n + (size_t)y * n + x));
+            v = load4(u + smp * (size_t)n * n + (size_t)y * n + x, wide);
         }
         *reinterpret_cast<float4 *>(dst + smp * (size_t)P * P + (size_t)py * P + px) = v;
     }
@@ -936,8 +972,7 @@ mfmc_status run_solve(Model &m, int algo, const StepCoef *coef, const float *u0,
     const bool constant = m.d.kernel == MFMC_KERNEL_CONSTANT;
     const TileLauncher *L = tile_launcher(m.R);
     const int ai = algo == MFMC_ALGO_DIRECT ? 0 : 1;
-    const bool tiled =
-        algo != MFMC_ALGO_PLAIN && constant && L && L->fn[ai] && m.d.bc == MFMC_BC_PERIODIC && m.integer_R;
+    const bool tiled = tiled_form(m, algo);
 
     if (algo == MFMC_ALGO_PLAIN) {
         // reference form: one sample per launch, one launch per step

@@ -85,6 +85,8 @@ extern "C" mfmc_status mfmc_solve_fields_noalloc(const mfmc_model *cm, const dou
     if (ns == 0) return MFMC_OK;
     if (!u0) return fail(MFMC_EINVAL, "NULL u0");
     if (uT && uT == u0) return fail(MFMC_EINVAL, "uT must not alias u0");
+    if ((uintptr_t)u0 % 16 || (uintptr_t)uT % 16)  // (its kernel's accesses; there is no scratch for a copy)
+        return fail(MFMC_EINVAL, "the allocation-free solve needs u0 and uT on 16-byte boundaries");
     const Model &m = *cm;
     const TileLauncher *L = tile_launcher(m.R);
     if (m.d.kernel != MFMC_KERNEL_CONSTANT || m.d.bc != MFMC_BC_PERIODIC || !m.integer_R || m.d.beta2 > 0.0 || !L)
