@@ -75,18 +75,20 @@ typedef enum {
     MFMC_ALGO_DIRECT = 1,      /* sum over every disc point                       */
     MFMC_ALGO_PREFIX = 2,      /* in-register row prefix sums: O(R) adds per point */
     MFMC_ALGO_PREFIX_KAHAN = 3,/* prefix form with compensated accumulation       */
-    MFMC_ALGO_RESIDENT = 4,    /* whole field held on chip for all steps (AUTO and the
-                                  server also run n = 256 this way, in clusters of CTAs) */
+    MFMC_ALGO_RESIDENT = 4,    /* whole field held on chip for all steps (constant kernel;
+                                  n % 16 == 0 and n <= 128 with R in {1,2,3,4,5,6,8}, n = 256
+                                  with R in {4,6,8} in clusters of four CTAs)     */
     MFMC_ALGO_PLAIN = 5,       /* reference form: one sample per launch, direct   */
     MFMC_ALGO_PREFIX_TMA = 6,  /* prefix form, persistent CTAs, TMA double-buffered
                                   tiles of a ghost-framed field                   */
     MFMC_ALGO_ROWS = 7         /* row streaming: one CTA per SM walks its share of the
-                                  batch's rows (groups of 2048/n samples) down through a ring of
-                                  TMA chunks of whole rows; a warp takes a 128-column strip
-                                  of one sample, a lane 4 columns with a ring of 2R+1
-                                  accumulators, every staged row summed once per segment
-                                  (constant kernel, R in {2,4,6,8}, n % 128 == 0; AUTO also
-                                  runs it at R = 12 and 16)  */,
+                                  batch's rows (groups of 2048/n samples, 1536/n at R = 12,
+                                  1024/n at R = 16) down through a ring of TMA chunks of whole
+                                  rows; a warp takes a 128-column strip of one sample, a lane
+                                  4 columns with 2R+1 accumulators that shift by one output row
+                                  per staged row, every staged row summed once per segment
+                                  (constant kernel, n % 128 == 0; R in {2,4,6,8}, R = 12 with
+                                  n <= 640, R = 16 with n = 128, 256, 512 or 1024)  */,
     MFMC_ALGO_FFT = 8          /* spectral form of the disc sum: cuFFT transforms (a library,
                                   loaded at run time) of each field, a product with the
                                   transform of the disc weights and the fused update; cost
@@ -169,7 +171,11 @@ typedef struct {
     int disc_points;       /* |D| = #{z in Z^2 : |z| <= R}                          */
     double c_gamma;        /* sum_z h^2 gamma(|z| h), the lattice c_gamma           */
     double xi;             /* c_gamma - c_F, Eq. (xi_constant)                      */
-    int algo;              /* mfmc_algo the solver uses for this model             */
+    int algo;              /* mfmc_algo the solver uses for this model: the name given, or
+                              AUTO's choice once a solve has made it, which can be given as a
+                              name in any process.  Where that is MFMC_ALGO_ROWS, AUTO runs a
+                              batch with fewer than 4R rows for each SM by PREFIX_TMA, whose
+                              fields have the same bits (rows of its sample groups)  */
     size_t field_bytes;    /* n * n * 4                                             */
     int tile_variant;      /* tile shape of the TMA kernel (0..10) the solver uses */
     int band_height;       /* rows per work range of the row-streaming kernel

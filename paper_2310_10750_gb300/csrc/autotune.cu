@@ -35,14 +35,6 @@ static std::tuple<int, int, int, int, int> tune_key(const Model &m) {
     return std::make_tuple(m.d.n, m.R, (int)m.d.kernel, (int)m.d.bc, m.r2max);
 }
 
-bool algo_selectable(const Model &m, int algo) {
-    if (!algo_supported(m, algo)) return false;
-    if (!(algo == MFMC_ALGO_ROWS && m.R > 8) && !(algo == MFMC_ALGO_RESIDENT && m.d.n > 128)) return true;
-    std::lock_guard<std::mutex> lk(g_tune_mu);
-    auto it = g_tune_cache.find(tune_key(m));
-    return it != g_tune_cache.end() && it->second.algo == algo;
-}
-
 mfmc_status autotune(Model &m, cudaStream_t st) {
     if (m.d.beta2 > 0.0) {  // one solver serves beta2 > 0
         m.algo = MFMC_ALGO_ACTIVE_SET;

@@ -221,7 +221,7 @@ mfmc_status mfmc_model_create(const mfmc_model_desc *desc, mfmc_model **out) {
             m->wsq[(size_t)dy * (R + 1) + dx] = desc->kernel == MFMC_KERNEL_CONSTANT ? 1.f : m->wtab[dx * dx + dy * dy];
     m->algo = desc->algo;
     m->tuned = 0;
-    if (m->algo != MFMC_ALGO_AUTO && !algo_selectable(*m, m->algo)) {
+    if (m->algo != MFMC_ALGO_AUTO && !algo_supported(*m, m->algo)) {
         delete m;
         return fail(MFMC_EINVAL, "algorithm %d does not support this model (R=%d, kernel=%d)", (int)desc->algo, R,
                     (int)desc->kernel);
@@ -398,7 +398,7 @@ static mfmc_status solve_impl(mfmc_model *m, int algo, const double *eps, const 
         }
         algo = m->algo;
         if (algo == MFMC_ALGO_ROWS && rows_batch_short(*m, ns)) algo = MFMC_ALGO_PREFIX_TMA;
-    } else if (!algo_selectable(*m, algo)) {
+    } else if (!algo_supported(*m, algo)) {
         return fail(MFMC_EINVAL, "algorithm %d does not support this model", algo);
     }
     const size_t nn = (size_t)m->d.n * m->d.n;

@@ -261,13 +261,9 @@ mfmc_status run_solve_active_set(Model &m, const double *eps_dev, const float *u
 // passes such fields through aligned copies when they do not start on a 16-byte boundary.
 bool wide_u0(const Model &m, int algo);
 bool wide_uT(const Model &m, int algo);
-// Whether an algorithm can run this model.
+// Whether an algorithm can run this model: what a caller may name and what AUTO considers, so that the
+// algorithm mfmc_model_query reports can always be asked for.  It depends on the descriptor alone.
 bool algo_supported(const Model &m, int algo);
-// Whether a caller may name it for this model.  The row kernel's R = 12 and 16 and the resident form's
-// n = 256 are AUTO's (and the server's) choice: a caller may name them once AUTO has chosen them for
-// the lattice and horizon in this process, so that the algorithm mfmc_model_query reports can be
-// asked for.
-bool algo_selectable(const Model &m, int algo);
 // Autotuner: time the candidate algorithms on this model once and cache the winner.
 mfmc_status autotune(Model &m, cudaStream_t st);
 

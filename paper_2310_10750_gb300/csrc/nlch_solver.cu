@@ -802,12 +802,22 @@ mfmc_status rows_alloc_buffers(const Model &m, int bh, size_t ns, TmaBuffers *b,
     return encode_rows_maps(b, m, g, L->ch);
 }
 
+// The lattices of the long horizons.  R = 16: those whose rows fill a CTA's eight warps; where warps stay
+// idle the tile kernel is the faster one (16 steps timed by the autotuner at n = 384, 640, 768, 896).
+// R = 12: n <= 640 (us a step, row and tile kernel: 256^2, 1024 samples 186 and 224; 512^2, 256 188 and
+// 231; 640^2, 163 197 and 220; at n = 1024 the tile kernel wins, and at n = 768, 191 and 219, the name
+// is refused as it always was, so AUTO does not take what it could not report).
+static bool rows_long_reach(int n, int R) {
+    if (R <= 8) return true;
+    return R == 16 ? 1024 % n == 0 : n <= 640;
+}
+
 // The row-streaming kernel: constant kernel, periodic lattice, integer R, 128-column strips (at most
 // one CTA's warps of them a row), four columns per thread.
 bool rows_supported(const Model &m, int rx) {
     RowsGeom g;
     return m.d.kernel == MFMC_KERNEL_CONSTANT && m.d.bc == MFMC_BC_PERIODIC && m.integer_R && rx == 4 &&
-           rows_launcher(m.R) != nullptr && rows_geom(m, &g);
+           rows_launcher(m.R) != nullptr && rows_geom(m, &g) && rows_long_reach(m.d.n, m.R);
 }
 
 // Whether a batch is too short for the row-streaming kernel: a CTA then walks 2R halo rows for few
