@@ -248,7 +248,9 @@ mfmc_status mfmc_model_solver_stats(const mfmc_model *model, uint64_t *newton_it
 mfmc_status mfmc_model_set_iteration_limits(mfmc_model *model, int newton_max, int cg_max);
 
 /* Pin the tile shape (0..10) of the TMA kernel instead of letting the autotuner choose
- * (for measurements and tests).  MFMC_EINVAL for an unknown variant. */
+ * (for measurements and tests).  The shape holds for solves that name MFMC_ALGO_PREFIX_TMA and for
+ * the server; where AUTO chooses that kernel itself it also chooses the shape.  MFMC_EINVAL for an
+ * unknown variant. */
 mfmc_status mfmc_model_set_tile_variant(mfmc_model *model, int variant);
 
 /* Pin the work split of the row-streaming kernel: rows = rows per work range (>= 8; the

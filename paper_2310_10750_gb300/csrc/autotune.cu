@@ -23,7 +23,9 @@ static std::map<std::tuple<int, int, int, int, int>, Tuned> g_tune_cache;
 
 static void apply(Model &m, const Tuned &t) {
     m.algo = t.algo;
-    if (t.tile >= 0) m.tma_variant = t.tile;  // also for batches too short for the row kernel
+    m.tile_fastest = t.tile;
+    // a pinned shape gives way only where the tile kernel is the choice
+    if (t.algo == MFMC_ALGO_PREFIX_TMA || (t.tile >= 0 && !m.tile_pinned)) m.tma_variant = t.tile;
     if (t.algo == MFMC_ALGO_ROWS) {
         m.rows_bh = t.param / 8;
         m.rows_rx = t.param % 8;

@@ -269,6 +269,7 @@ mfmc_status mfmc_model_set_tile_variant(mfmc_model *m, int variant) {
     if (!m || variant < 0 || variant >= kTmaVariants) return fail(MFMC_EINVAL, "invalid tile variant");
     std::lock_guard<std::mutex> lk(m->mu);
     m->tma_variant = variant;
+    m->tile_pinned = 1;
     return MFMC_OK;
 }
 
@@ -321,8 +322,9 @@ mfmc_status mfmc_init_fields(const mfmc_model *cm, const mfmc_sample_params *par
     return MFMC_OK;
 }
 
-// The solve by one algorithm, the model's lock held, u0 and uT aligned as its kernels need.
-static mfmc_status solve_by(mfmc_model *m, int algo, const double *eps, const float *u0, size_t ns, float *uT,
+// The solve by one algorithm (variant: tile shape of PREFIX_TMA), the model's lock held, u0 and uT
+// aligned as its kernels need.
+static mfmc_status solve_by(mfmc_model *m, int algo, int variant, const double *eps, const float *u0, size_t ns, float *uT,
                             double *ubar, double *ooi, cudaStream_t st, int nsteps) {
     if (algo == MFMC_ALGO_ACTIVE_SET) return run_solve_active_set(*m, eps, u0, ns, nsteps, uT, ubar, ooi, st);
     mfmc_status s = grow(&m->coef, &m->coef_cap, ns);
@@ -337,7 +339,7 @@ static mfmc_status solve_by(mfmc_model *m, int algo, const double *eps, const fl
     const bool graphable = !m->graphs_off && algo != MFMC_ALGO_RESIDENT && algo != MFMC_ALGO_PLAIN &&
                            algo != MFMC_ALGO_FFT && nsteps > 0;
     auto key = [&]() {
-        return std::vector<uintptr_t>{(uintptr_t)algo, (uintptr_t)m->tma_variant, (uintptr_t)m->rows_bh,
+        return std::vector<uintptr_t>{(uintptr_t)algo, (uintptr_t)variant, (uintptr_t)m->rows_bh,
                                       (uintptr_t)m->rows_rx, (uintptr_t)ns, (uintptr_t)nsteps, (uintptr_t)eps,
                                       (uintptr_t)u0, (uintptr_t)uT, (uintptr_t)ubar, (uintptr_t)ooi,
                                       (uintptr_t)st, (uintptr_t)m->coef, (uintptr_t)m->bufA, (uintptr_t)m->bufB,
@@ -351,7 +353,7 @@ static mfmc_status solve_by(mfmc_model *m, int algo, const double *eps, const fl
     }
     s = launch_coefficients(*m, eps, ns, m->coef, st);
     if (s != MFMC_OK) return s;
-    s = run_solve(*m, algo, m->coef, u0, ns, nsteps, uT, ubar, ooi, st);
+    s = run_solve(*m, algo, m->coef, u0, ns, nsteps, uT, ubar, ooi, st, variant);
     if (s != MFMC_OK || !graphable) return s;
     if (m->gexec) {
         cudaGraphExecDestroy(m->gexec);
@@ -364,7 +366,7 @@ static mfmc_status solve_by(mfmc_model *m, int algo, const double *eps, const fl
         return MFMC_OK;
     }
     mfmc_status cs = launch_coefficients(*m, eps, ns, m->coef, st);
-    if (cs == MFMC_OK) cs = run_solve(*m, algo, m->coef, u0, ns, nsteps, uT, ubar, ooi, st);
+    if (cs == MFMC_OK) cs = run_solve(*m, algo, m->coef, u0, ns, nsteps, uT, ubar, ooi, st, variant);
     cudaError_t e = cudaStreamEndCapture(st, &g);
     if (cs == MFMC_OK && e == cudaSuccess && g) e = cudaGraphInstantiate(&m->gexec, g, 0);
     if (g) cudaGraphDestroy(g);
@@ -391,13 +393,18 @@ static mfmc_status solve_impl(mfmc_model *m, int algo, const double *eps, const 
         return fail(MFMC_EINVAL, "u0 and uT must be aligned as floats");
     if (ns > (size_t)kMaxNs) return fail(MFMC_EINVAL, "too many samples");
     std::lock_guard<std::mutex> lk(m->mu);
+    int variant = m->tma_variant;
     if (algo == MFMC_ALGO_AUTO) {
         if (!m->tuned) {
             mfmc_status s = autotune(*m, st);
             if (s != MFMC_OK) return s;
         }
         algo = m->algo;
-        if (algo == MFMC_ALGO_ROWS && rows_batch_short(*m, ns)) algo = MFMC_ALGO_PREFIX_TMA;
+        variant = m->tma_variant;
+        if (algo == MFMC_ALGO_ROWS && m->tile_fastest >= 0 && rows_batch_short(*m, ns)) {
+            algo = MFMC_ALGO_PREFIX_TMA;
+            variant = m->tile_fastest;
+        }
     } else if (!algo_supported(*m, algo)) {
         return fail(MFMC_EINVAL, "algorithm %d does not support this model", algo);
     }
@@ -414,7 +421,7 @@ static mfmc_status solve_impl(mfmc_model *m, int algo, const double *eps, const 
         mfmc_status s = grow_buffer(&m->uT_copy, &m->uT_copy_cap, ns * nn);
         if (s != MFMC_OK) return s;
     }
-    mfmc_status s = solve_by(m, algo, eps, u0, ns, copy_out ? m->uT_copy : uT, ubar, ooi, st, nsteps);
+    mfmc_status s = solve_by(m, algo, variant, eps, u0, ns, copy_out ? m->uT_copy : uT, ubar, ooi, st, nsteps);
     if (s == MFMC_OK && copy_out)
         MFMC_CUDA(cudaMemcpyAsync(uT, m->uT_copy, ns * nn * sizeof(float), cudaMemcpyDeviceToDevice, st));
     return s;

@@ -91,6 +91,8 @@ struct Model {
     int maps_valid = 0;
     int map_sw = 0, map_sh = 0, map_sd = 1, map_l2 = 256;  // box and L2 promotion of the tensor maps
     int tma_variant = 4;         // tile shape of the TMA kernel (autotuned; 4 is the default)
+    int tile_pinned = 0;         // set by mfmc_model_set_tile_variant
+    int tile_fastest = -1;       // the fastest shape AUTO timed: short batches of a row-streaming lattice
     int rows_bh = 0;             // rows per work range of the row-streaming kernel (0: even split)
     int rows_rx = 4;             // columns per thread of the row-streaming kernel
     int *d_status = nullptr;  // set by a device wait that gave up
@@ -176,8 +178,9 @@ mfmc_status launch_init_fields(const Model &m, const uint64_t *seeds_dev,
 mfmc_status launch_coefficients(const Model &m, const double *eps_dev, size_t ns,
                                 StepCoef *coef, cudaStream_t st);
 // Full solve with an explicit algorithm; scratch from the model.
+// variant: tile shape of PREFIX_TMA, or -1 for the model's.
 mfmc_status run_solve(Model &m, int algo, const StepCoef *coef, const float *u0, size_t ns,
-                      int nsteps, float *uT, double *ubar, double *ooi, cudaStream_t st);
+                      int nsteps, float *uT, double *ubar, double *ooi, cudaStream_t st, int variant = -1);
 // Buffers of one run of the TMA pipeline (model scratch, or a serving cohort's own).
 struct TmaBuffers {
     float *padA = nullptr, *padB = nullptr;

@@ -951,7 +951,7 @@ mfmc_status run_resident_steps(const Model &m, const StepCoef *coef, const float
 }
 
 mfmc_status run_solve(Model &m, int algo, const StepCoef *coef, const float *u0, size_t ns, int nsteps,
-                      float *uT, double *ubar, double *ooi, cudaStream_t st) {
+                      float *uT, double *ubar, double *ooi, cudaStream_t st, int variant) {
     if (ns == 0) return MFMC_OK;
     const int n = m.d.n;
     const size_t nn = (size_t)n * n;
@@ -970,7 +970,7 @@ mfmc_status run_solve(Model &m, int algo, const StepCoef *coef, const float *u0,
     if (algo == MFMC_ALGO_SPECTRAL) return run_solve_spectral(m, coef, u0, ns, nsteps, uT, ubar, ooi, st);
     if (algo == MFMC_ALGO_WEIGHTED) return run_solve_tma(m, 0, kTmaWeighted, coef, u0, ns, nsteps, uT, ubar, ooi, st);
     if (algo == MFMC_ALGO_PREFIX_TMA)
-        return run_solve_tma(m, 0, m.tma_variant, coef, u0, ns, nsteps, uT, ubar, ooi, st);
+        return run_solve_tma(m, 0, variant < 0 ? m.tma_variant : variant, coef, u0, ns, nsteps, uT, ubar, ooi, st);
     if (algo == MFMC_ALGO_PREFIX_KAHAN) return run_solve_tma(m, 1, 0, coef, u0, ns, nsteps, uT, ubar, ooi, st);
     if (algo == MFMC_ALGO_ROWS) return run_solve_rows(m, m.rows_bh, 4, coef, u0, ns, nsteps, uT, ubar, ooi, st);
     if (algo == MFMC_ALGO_RESIDENT) return run_resident_steps(m, coef, u0, ns, nsteps, nullptr, uT, ubar, ooi, st);
