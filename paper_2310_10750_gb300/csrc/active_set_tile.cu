@@ -33,6 +33,7 @@ namespace mfmc {
 
 namespace {
 
+constexpr int AT_SPARE_PASSES = 40;  // of the default bound's 60; a step takes 4 to 8
 constexpr int AT_NU_COARSE = 8;  // coarsest sweeps (16, as the fallback kernel has: no CG iteration fewer)
 
 template <int N>
@@ -632,9 +633,12 @@ __global__ void __launch_bounds__(AtCfg<N>::NT, MINB) active_set_tile_kernel(con
                 for (int c = 0; c < CW; ++c) f[y][c] *= sc;
             // CG on J d = f from d = 0, preconditioned by one V-cycle, to a residual that matches what the
             // correction can be worth: while the active set still moves it limits the next residual, not
-            // the solve, and on a settled set the next residual is this one times the tolerance (1e-5
-            // throughout: 33.1 CG iterations a step of 128^2 samples, now 26.1)
-            const float rtol = it == 1 ? 3e-2f : (changed ? 1e-3f : 1e-6f);
+            // the solve, and on a settled set the next residual is this one times the tolerance (AS_CG_RTOL
+            // throughout: 33.1 CG iterations a step of 128^2 samples, now 26.1).  The loose corrections
+            // cost a pass here and there (4.8 -> 5.1), so they are left to steps with passes to spare: under
+            // a caller's tighter bound, and late in a step, every correction is worth its pass.
+            const bool spare = a.newton_max - it >= AT_SPARE_PASSES;
+            const float rtol = spare && it == 1 ? 3e-2f : (spare && changed ? 1e-3f : (changed || it == 1 ? AS_CG_RTOL : 1e-6f));
             float rz = 0.0f;
             for (int k = 1;; ++k) {
                 float v[RW][CW];

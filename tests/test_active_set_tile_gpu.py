@@ -55,3 +55,25 @@ def test_one_non_finite_value_stops_its_sample_alone(gpu_lib, n, value):
     assert np.all(vT[1] == 7.0) and voi[1] == 7.0
     for i in (0, 2):
         assert np.array_equal(vT[i], uT[i]) and voi[i] == ooi[i]
+
+
+# The passes that steps of these samples take with every correction solved to 1e-5, the tolerance of the
+# kernel for other lattices: a caller's bound of as many passes is enough.
+@pytest.mark.parametrize("n,delta,kernel,steps,ns,passes", [
+    (64, 4 / 64, 0, 10, 20, 5), (64, 0.125, 1, 10, 20, 6), (64, 0.25, 1, 10, 20, 6), (88, 0.1875, 1, 8, 12, 6),
+    (128, 0.25, 1, 6, 12, 6), (128, 0.0625, 1, 6, 12, 7)])
+def test_a_tight_pass_bound_is_met(gpu_lib, n, delta, kernel, steps, ns, passes):
+    mf = gpu_lib
+    g = mf.Model(n=n, delta=delta, kernel=kernel, delta_hf=0.25 if kernel else 0.0, eps=0.04219, tau=0.01,
+                 nsteps=steps, ic=2, beta2=0.05)
+    seeds = np.arange(ns, dtype=np.uint64) + 50
+    free, _ = mf.mfmc_solve_batch([g] * ns, seeds)
+    g.set_iteration_limits(newton_max=passes)
+    bound, _ = mf.mfmc_solve_batch([g] * ns, seeds)
+    assert np.abs(bound - free).max() <= 1e-8  # both to max |F| <= 1e-11 a step
+    newton, _ = mf.mfmc_model_solver_stats(g)
+    assert newton <= passes * ns * steps
+    g.set_iteration_limits(newton_max=2)
+    with pytest.raises(mf.MfmcError) as e:
+        mf.mfmc_solve_batch([g] * ns, seeds)
+    assert e.value.status == mf.MFMC_ETIMEOUT
