@@ -380,17 +380,21 @@ __device__ __noinline__ void sq_solve_generic(const SqModelDev &M, int s, float 
                 u[y * n + x] = fminf(1.f, fmaxf(-1.f, v));
             });
     __syncthreads();
-    double acc = 0.0;
-    for (int i = threadIdx.x; i < nn; i += blockDim.x) {
-        const float x = u[i];
-        acc += (double)x;
-        if (M.uT) M.uT[(size_t)s * nn + i] = x;
+    // summed by the first kSqThreads threads whatever the CTA has, so that the mean does not depend on
+    // which lattices share the launch
+    if (threadIdx.x < kSqThreads) {
+        double acc = 0.0;
+        for (int i = threadIdx.x; i < nn; i += kSqThreads) {
+            const float x = u[i];
+            acc += (double)x;
+            if (M.uT) M.uT[(size_t)s * nn + i] = x;
+        }
+        red[threadIdx.x] = acc;
     }
-    red[threadIdx.x] = acc;
     __syncthreads();
     if (threadIdx.x == 0) {
         double tot = 0.0;
-        for (int i = 0; i < (int)blockDim.x; ++i) tot += red[i];
+        for (int i = 0; i < kSqThreads; ++i) tot += red[i];
         const double mean = tot / (double)nn;
         if (M.ubar) M.ubar[s] = mean;
         if (M.ooi) M.ooi[s] = 0.5 * (1.0 + mean);
