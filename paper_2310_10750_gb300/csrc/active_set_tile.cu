@@ -18,7 +18,7 @@
 // What bounds it: the fallback kernel (fine-level vectors in L2, generic indices) issued 943
 // instructions per point and CG iteration, and waited on L2 (long scoreboard 4.4 cycles an
 // instruction).  Here the FP64 pipe (two lanes a clock an SM) takes the larger part of a step:
-// the disc sum's transforms (444 K cycles a step of 128^2) and 8 operations per point of a Newton
+// the disc sum's transforms (444 K cycles a step of 128^2) and 7 operations per point of a Newton
 // residual (88 K); a V-cycle is 21 K cycles.  beta2 = 0.05: 50 samples of 128^2, 20 steps, 17.1 ms
 // (fallback kernel 113), 1000 of 64^2, 10 steps, 11.2 ms (106), 304 of 88^2, 8 steps, 8.4 ms.
 #include <cuda_runtime.h>
@@ -52,6 +52,12 @@ struct AtCfg {
     static_assert(LU <= 32 && N % RW == 0 && N % CW == 0, "one warp per row block");
 };
 
+// a / b rounded to nearest, from r = 1 / b rounded to nearest: one correction of the product a r by its
+// exact remainder (Markstein, IBM J. Res. Dev. 34, 1990), three operations where a division takes about ten.
+__device__ __forceinline__ double at_div(double a, double b, double r) {
+    const double q = a * r;
+    return fma(fma(-q, b, a), r, q);
+}
 __device__ __forceinline__ double at_clip(double v) { return v > 1.0 ? 1.0 : (v < -1.0 ? -1.0 : v); }
 
 template <int C>
@@ -529,7 +535,10 @@ __global__ void __launch_bounds__(AtCfg<N>::NT, MINB) active_set_tile_kernel(con
     const double eps = a.eps ? a.eps[smp] : a.eps_nominal;
     const double e2a = eps * eps * a.ahat, cg = e2a * a.chat, icg = 1.0 / cg;
     const double tb1 = a.tau * a.beta1, tb2h = a.tau * a.beta2 * (double)N * (double)N;
-    const double wdiag = tb1 + 4.0 * tb2h;
+    // the residual is formed as c_gamma F = (c_gamma tau A) w + P_[-c_gamma, c_gamma](w + g) - c_gamma u:
+    // no quotient, and one operation fewer than with the product by 1 / c_gamma
+    const double cgtb2 = cg * tb2h, cgdiag = fma(4.0, cgtb2, cg * tb1), ftol = 1e-11 * cg;
+    const unsigned long long cgbits = (unsigned long long)__double_as_longlong(cg);
     t.tb1 = (float)tb1;
     t.icg = (float)icg;
     t.tb2 = (float)tb2h;
@@ -574,9 +583,10 @@ __global__ void __launch_bounds__(AtCfg<N>::NT, MINB) active_set_tile_kernel(con
         }
         for (int it = 1;; ++it) {
             ++n_newton;
-            // FP64 residual F(w), the inactive set, and the right-hand side f = -F of J d = -F
+            // FP64 residual c_gamma F(w), the inactive set, and the right-hand side of J d = -F, which is
+            // f = -(c_gamma F) / max |c_gamma F| with d scaled back by max |c_gamma F| / c_gamma
             float f[RW][CW];
-            unsigned fhi = 0u;  // maximum of the high words of |F|: a NaN's lies above every number's
+            unsigned fhi = 0u;  // maximum of the high words of |c_gamma F|: a NaN's lies above every number's
             unsigned now = 0u;
             {
                 double up[CW], cur[CW], dn[CW];
@@ -595,12 +605,12 @@ __global__ void __launch_bounds__(AtCfg<N>::NT, MINB) active_set_tile_kernel(con
                     for (int c = 0; c < CW; ++c) {
                         const double S = (up[c] + dn[c]) + ((c == 0 ? l : cur[c > 0 ? c - 1 : 0]) +
                                                             (c == CW - 1 ? r : cur[c + 1 < CW ? c + 1 : c]));
-                        const double xv = (cur[c] + g[c]) * icg;
-                        // |x| < 1 and the projection from the exponent bits (no FP64 compares)
-                        const int hi = __double2hiint(xv);
-                        const bool in = (hi & 0x7fffffff) < 0x3ff00000;
-                        const double xc = in ? xv : __hiloint2double((hi & 0x80000000) | 0x3ff00000, 0);
-                        const double F = fma(wdiag, cur[c], fma(-tb2h, S, xc - u[c]));
+                        const double z = cur[c] + g[c];
+                        // |z| < c_gamma and the projection on the bit patterns (no FP64 compares)
+                        const unsigned long long zb = (unsigned long long)__double_as_longlong(z);
+                        const bool in = (zb & ~(1ull << 63)) < cgbits;
+                        const double zc = in ? z : __longlong_as_double((long long)((zb & 1ull << 63) | cgbits));
+                        const double F = fma(cgdiag, cur[c], fma(-cgtb2, S, fma(-cg, u[c], zc)));
                         now |= in ? 1u << (y * CW + c) : 0u;
                         f[y][c] = act ? -(float)F : 0.0f;
                         fhi = umax(fhi, (unsigned)__double2hiint(F) & 0x7fffffffu);
@@ -614,9 +624,9 @@ __global__ void __launch_bounds__(AtCfg<N>::NT, MINB) active_set_tile_kernel(con
             }
             const bool changed = __syncthreads_or(act && now != t.mask);
             t.mask = now;
-            // the largest |F| with that high word: what passes meets the bound in full
+            // the largest value with that high word: what passes meets the bound in full
             const double fbound = __hiloint2double((int)t.max_bits(act ? fhi : 0u), -1);
-            if (it > 1 && !changed && fbound <= 1e-11) break;
+            if (it > 1 && !changed && fbound <= ftol) break;
             // the bound on the passes, or a residual that no pass mends (a NaN or an infinity, which the
             // correction would carry to every point): the sample's solve stops
             if (it > a.newton_max || !(fbound < INFINITY)) {
@@ -708,7 +718,7 @@ __global__ void __launch_bounds__(AtCfg<N>::NT, MINB) active_set_tile_kernel(con
                 }
             }
             if (act) {
-                const double scale = (double)fmax;
+                const double scale = (double)fmax * icg;
 #pragma unroll
                 for (int y = 0; y < RW; ++y) {
                     double w[CW];
@@ -728,7 +738,7 @@ __global__ void __launch_bounds__(AtCfg<N>::NT, MINB) active_set_tile_kernel(con
                 at_ld64<CW>(w, W + own + y * N);
                 at_ld64<CW>(g, G + own + y * N);
 #pragma unroll
-                for (int c = 0; c < CW; ++c) w[c] = at_clip((w[c] + g[c]) * icg);
+                for (int c = 0; c < CW; ++c) w[c] = at_clip(at_div(w[c] + g[c], cg, icg));
                 at_st64<CW>(U + own + y * N, w);
             }
         }
