@@ -45,10 +45,14 @@ struct AtCfg {
     static constexpr int LEVELS = CW == 4 ? 3 : 2;  // levels held in registers: CW >> level columns a lane
     static constexpr int TN = N >> LEVELS;          // the first level of the one-warp part
     static constexpr int XP = 32 * CW;              // floats of an exchanged row
-    // shared memory (floats): p, q, the exchange rows (two buffers of two rows a warp), then the
-    // one-warp part's right-hand side, diagonal and result
+    // shared memory (floats): p, q, the exchange rows (two buffers of two rows a warp), the one-warp
+    // part's right-hand side, result, diagonal, relaxation factors and 8^2 factors, then the relaxation
+    // factors of levels 1 and 2
     static constexpr int P = 0, Q = N * N, X = 2 * N * N, T = X + 4 * NW * XP;
-    static constexpr size_t SMEM = (size_t)(T + 3 * TN * TN) * sizeof(float);
+    static constexpr int RX1 = T + (4 * TN * TN + 64), RX2 = RX1 + N * N / 4;
+    // N = 64 forms them in every sweep: four CTAs an SM bind on shared memory (11.45 ms held, 11.34 formed)
+    static constexpr bool HOLD = N != 64;
+    static constexpr size_t SMEM = (size_t)(HOLD ? RX2 + N * N / 16 : RX1) * sizeof(float);
     static_assert(LU <= 32 && N % RW == 0 && N % CW == 0, "one warp per row block");
 };
 
@@ -112,6 +116,7 @@ struct At {
     using K = AtCfg<N>;
     float *sm, *red;
     int warp, lane, left, right;  // lanes of the columns left and right of the lane's (periodic)
+    int slot;                     // the lane's first column in a [row][warp][lane] layout (idle lanes: lane 0's)
     int par, rpar;                // the exchange and reduction buffers in turn
     unsigned mask;                // inactive set: bit row * CW + column
     float tb1, icg, tb2;          // tb2: level 0; level l has tb2 / 4^l
@@ -190,12 +195,41 @@ struct At {
         else
             return fmaf((float)__popc(mask & bits<L>(y, c)), icg * (1.0f / (1 << (2 * L))), d);
     }
+    // omega / diagonal of the lane's row y of level L.  Those of levels 1 and 2 hold for a Newton pass:
+    // divided once (hold_relax) into shared memory, each thread reading back its own.
     template <int L>
-    __device__ __forceinline__ float relax(int y, int c) const {  // omega / diagonal
-        if constexpr (L == 0)
-            return (mask & bits<0>(y, c)) ? w1 : w0;
-        else
-            return __fdividef(AS_OMEGA, diag<L>(y, c));
+    __device__ __forceinline__ float *relax_at(int y) const {
+        return sm + (L == 1 ? K::RX1 : K::RX2) + y * (K::NW * K::LU * (K::CW >> L)) + (slot >> L);
+    }
+    template <int L, int C>
+    __device__ __forceinline__ void relax(int y, float (&w)[C]) const {
+        static_assert(C == K::CW >> L, "a level's columns");
+        if constexpr (L == 0) {
+#pragma unroll
+            for (int c = 0; c < C; ++c) w[c] = (mask & bits<0>(y, c)) ? w1 : w0;
+        } else if constexpr (K::HOLD) {
+            at_ld<C>(w, relax_at<L>(y));
+        } else {
+#pragma unroll
+            for (int c = 0; c < C; ++c) {  // the fast quotient corrected by its remainder
+                const float d = diag<L>(y, c), r = __fdividef(1.0f, d), q = AS_OMEGA * r;
+                w[c] = fmaf(fmaf(-q, d, AS_OMEGA), r, q);
+            }
+        }
+    }
+    template <int L>
+    __device__ __forceinline__ void hold_relax() {
+        constexpr int C = K::CW >> L;
+        if (lane < K::LU) {
+#pragma unroll
+            for (int y = 0; y < (K::RW >> L); ++y) {
+                float w[C];
+#pragma unroll
+                for (int c = 0; c < C; ++c) w[c] = AS_OMEGA / diag<L>(y, c);
+                at_st<C>(relax_at<L>(y), w);
+            }
+        }
+        if constexpr (L + 1 < K::LEVELS) hold_relax<L + 1>();
     }
 };
 
@@ -216,12 +250,13 @@ __device__ __forceinline__ void at_sweep(At<N> &t, const float (&f)[R][C], float
     const float tb2 = t.template tb2l<L>();
 #pragma unroll
     for (int y = 0; y < R; ++y) {
-        float S[C];
+        float S[C], w[C];
         at_nb<N, C>(t, prev, v[y], y == R - 1 ? below : v[y + 1 < R ? y + 1 : y], S);
+        t.template relax<L, C>(y, w);
 #pragma unroll
         for (int c = 0; c < C; ++c) {
             prev[c] = v[y][c];
-            v[y][c] = fmaf(t.template relax<L>(y, c), fmaf(tb2, S[c], f[y][c]), (1.0f - AS_OMEGA) * v[y][c]);
+            v[y][c] = fmaf(w[c], fmaf(tb2, S[c], f[y][c]), (1.0f - AS_OMEGA) * v[y][c]);
         }
     }
 }
@@ -303,65 +338,58 @@ __device__ __forceinline__ void tail_sweep(const TailLanes<n> &p, const float (&
 
 template <int n>
 __device__ __forceinline__ void tail_coarsest(const TailLanes<n> &p, const float (&f)[TailCfg<n>::R],
-                                              const float (&d)[TailCfg<n>::R], float (&v)[TailCfg<n>::R], float tb2) {
-    float w[TailCfg<n>::R];
+                                              const float (&w)[TailCfg<n>::R], float (&v)[TailCfg<n>::R], float tb2) {
 #pragma unroll
-    for (int y = 0; y < TailCfg<n>::R; ++y) {
-        w[y] = __fdividef(AS_OMEGA, d[y]);
-        v[y] = w[y] * f[y];
-    }
+    for (int y = 0; y < TailCfg<n>::R; ++y) v[y] = w[y] * f[y];
 #pragma unroll 1
     for (int k = 2; k <= AT_NU_COARSE; ++k) tail_sweep<n>(p, f, w, v, tb2);
 }
 
-// One cycle from f to v (shared memory, n x n) by one warp; d: the diagonals.
+// One cycle of the n x n level by one warp.  fs (shared memory): the right-hand side, then the result,
+// the diagonals, omega / diagonal, and (n = 16) omega / diagonal of 8^2.
 template <int n>
-__device__ __noinline__ void tail_cycle(const float *fs, const float *ds, float *vs, float tb1, float tb2, int lane) {
+__device__ __noinline__ void tail_cycle(float *fs, float tb2, int lane) {
     constexpr int R = TailCfg<n>::R, G = TailCfg<n>::G;
     const TailLanes<n> p(lane);
-    float f[R], d[R], v[R];
+    float f[R], w[R], v[R];
 #pragma unroll
     for (int y = 0; y < R; ++y) {
         f[y] = fs[(p.g * R + y) * n + p.x];
-        d[y] = ds[(p.g * R + y) * n + p.x];
+        w[y] = fs[3 * n * n + (p.g * R + y) * n + p.x];
     }
     if constexpr (n != 16) {
-        tail_coarsest<n>(p, f, d, v, tb2);
+        tail_coarsest<n>(p, f, w, v, tb2);
     } else {  // 16^2 over 8^2: lane 16 g + x of 16^2 holds rows 8 g .., lane 8 g + x of 8^2 rows 2 g, 2 g + 1
         const TailLanes<8> q(lane);
-        float w[R], S[R], h[R], fc[2], dc[2], vc[2];
+        float d[R], S[R], h[R], fc[2], wc[2], vc[2];
 #pragma unroll
         for (int y = 0; y < R; ++y) {
-            w[y] = __fdividef(AS_OMEGA, d[y]);
             v[y] = w[y] * f[y];
         }
         tail_sweep<n>(p, f, w, v, tb2);
         tail_nb<n>(p, v, S);
+        asm volatile("" ::: "memory");  // the diagonals are not loaded earlier: registers
+#pragma unroll
+        for (int y = 0; y < R; ++y) d[y] = fs[2 * n * n + (p.g * R + y) * n + p.x];
 #pragma unroll
         for (int y = 0; y < R; ++y) {  // residual, weighted 1 2 1 along x
             const float r = fmaf(-d[y], v[y], fmaf(tb2, S[y], f[y]));
             h[y] = 0.25f * (tail_shfl(r, p.left) + tail_shfl(r, p.right)) + 0.5f * r;
         }
         const float ha = tail_shfl(h[R - 1], p.above);
-        // coarse rows 4 g' .. of this lane's column (g' = its half), then to the 8^2 owners; the coarse
-        // mean of m icg is the diagonals' mean less the stencil's part
-        float cf[R / 2], cd[R / 2];
-        const float s16 = tb1 + 4.0f * tb2, s8 = tb1 + tb2;
+        // coarse rows 4 g' .. of this lane's column (g' = its half), then to the 8^2 owners
+        float cf[R / 2];
 #pragma unroll
-        for (int Y = 0; Y < R / 2; ++Y) {
+        for (int Y = 0; Y < R / 2; ++Y)
             cf[Y] = 0.25f * ((Y == 0 ? ha : h[Y > 0 ? 2 * Y - 1 : 0]) + h[2 * Y + 1]) + 0.5f * h[2 * Y];
-            const float dd = d[2 * Y] + d[2 * Y + 1];
-            cd[Y] = 0.25f * (dd + tail_shfl(dd, p.right)) - s16 + s8;
-        }
         const int from = (q.g >> 1) * 16 + 2 * q.x;  // rows 2 q.g, 2 q.g + 1 = rows 2 (q.g & 1), + 1 of that half
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
             const float f0 = tail_shfl(cf[i], from), f1 = tail_shfl(cf[2 + i], from);
-            const float d0 = tail_shfl(cd[i], from), d1 = tail_shfl(cd[2 + i], from);
             fc[i] = (q.g & 1) ? f1 : f0;
-            dc[i] = (q.g & 1) ? d1 : d0;
+            wc[i] = fs[4 * n * n + (2 * q.g + i) * 8 + q.x];
         }
-        tail_coarsest<8>(q, fc, dc, vc, 0.25f * tb2);
+        tail_coarsest<8>(q, fc, wc, vc, 0.25f * tb2);
         // bilinear prolongation: coarse rows 4 g .. 4 g + 4 at columns x / 2 and (x odd) the next
         float e[R / 2 + 1];
         const int X = p.x >> 1, X1 = (p.x & 1) ? ((X + 1) & 7) : X;
@@ -379,7 +407,7 @@ __device__ __noinline__ void tail_cycle(const float *fs, const float *ds, float 
     }
     if (lane < G * n) {
 #pragma unroll
-        for (int y = 0; y < R; ++y) vs[(p.g * R + y) * n + p.x] = v[y];
+        for (int y = 0; y < R; ++y) fs[n * n + (p.g * R + y) * n + p.x] = v[y];
     }
 }
 
@@ -390,9 +418,12 @@ template <int N, int L, int C, int R>
 __device__ __forceinline__ void at_cycle(At<N> &t, const float (&f)[R][C], float (&v)[R][C]) {
     using K = AtCfg<N>;
 #pragma unroll
-    for (int y = 0; y < R; ++y)
+    for (int y = 0; y < R; ++y) {
+        float w[C];
+        t.template relax<L, C>(y, w);
 #pragma unroll
-        for (int c = 0; c < C; ++c) v[y][c] = t.template relax<L>(y, c) * f[y][c];
+        for (int c = 0; c < C; ++c) v[y][c] = w[c] * f[y][c];
+    }
     at_sweep<N, L, C, R>(t, f, v);
     constexpr int HC = C > 1 ? C / 2 : 1;
     float cf[R / 2][HC];
@@ -434,13 +465,13 @@ __device__ __forceinline__ void at_cycle(At<N> &t, const float (&f)[R][C], float
         }
     } else {
         constexpr int TN = K::TN;
-        float *tf = t.sm + K::T, *td = tf + TN * TN, *tv = td + TN * TN;
+        float *tf = t.sm + K::T, *tv = tf + TN * TN;
         if ((t.lane & 1) == 0 && t.lane < K::LU) {
 #pragma unroll
             for (int Y = 0; Y < R / 2; ++Y) tf[(t.warp * (R / 2) + Y) * TN + (t.lane >> 1)] = cf[Y][0];
         }
         __syncthreads();
-        if (t.warp == 0) tail_cycle<TN>(tf, td, tv, t.tb1, t.template tb2l<L + 1>(), t.lane);
+        if (t.warp == 0) tail_cycle<TN>(tf, t.template tb2l<L + 1>(), t.lane);
         __syncthreads();
         const int x = t.lane < K::LU ? t.lane : 0, X = x >> 1, X1 = (x & 1) ? (X + 1 == TN ? 0 : X + 1) : X;
 #pragma unroll
@@ -453,14 +484,15 @@ __device__ __forceinline__ void at_cycle(At<N> &t, const float (&f)[R][C], float
     at_sweep<N, L, C, R>(t, f, v);
 }
 
-// Diagonals of the first one-warp level from the threads' masks: the count over a 2^LEVELS square is
-// the lane's block of 2^LEVELS rows and the right lane's.
+// What holds of the one-warp levels for a Newton pass: the diagonals of the first from the threads'
+// masks (the count over a 2^LEVELS square is the lane's block of 2^LEVELS rows and the right lane's), and
+// the relaxation factors.
 template <int N>
-__device__ __forceinline__ void at_tail_diagonals(At<N> &t) {
+__device__ __forceinline__ void at_hold_tail(At<N> &t) {
     using K = AtCfg<N>;
     constexpr int TN = K::TN, LV = K::LEVELS, TR = K::RW >> LV;
     constexpr float area = 1.0f / (1 << (2 * LV));
-    float *td = t.sm + K::T + TN * TN;
+    float *td = t.sm + K::T + 2 * TN * TN, *tw = td + TN * TN, *tw8 = tw + TN * TN;
     const float d0 = t.tb1 + 4.0f * t.tb2 * area;
 #pragma unroll
     for (int Y = 0; Y < TR; ++Y) {
@@ -468,7 +500,17 @@ __device__ __forceinline__ void at_tail_diagonals(At<N> &t) {
                                                             : ((1u << ((K::CW << LV) & 31)) - 1u) << (Y * (K::CW << LV)));
         const int own = __popc(rows), both = own + __shfl_sync(0xffffffffu, own, t.right);
         if ((t.lane & 1) == 0 && t.lane < K::LU) {
-            td[(t.warp * TR + Y) * TN + (t.lane >> 1)] = fmaf((float)both, t.icg * area, d0);
+            const float d = fmaf((float)both, t.icg * area, d0);
+            td[(t.warp * TR + Y) * TN + (t.lane >> 1)] = d;
+            tw[(t.warp * TR + Y) * TN + (t.lane >> 1)] = AS_OMEGA / d;
+        }
+    }
+    if constexpr (TN == 16) {  // 8^2: the mean of m icg is the diagonals' mean less the stencil's part
+        __syncthreads();
+        if (threadIdx.x < 64) {
+            const float *d = td + (threadIdx.x >> 3) * 32 + (threadIdx.x & 7) * 2;
+            const float tb2 = t.tb2 * area, s16 = t.tb1 + 4.0f * tb2, s8 = t.tb1 + tb2;
+            tw8[threadIdx.x] = AS_OMEGA / (0.25f * ((d[0] + d[16]) + (d[1] + d[17])) - s16 + s8);
         }
     }
 }
@@ -521,15 +563,15 @@ __global__ void __launch_bounds__(AtCfg<N>::NT, MINB) active_set_tile_kernel(con
     t.warp = threadIdx.x >> 5;
     t.lane = threadIdx.x & 31;
     const bool act = t.lane < K::LU;
+    t.slot = (t.warp * K::LU + (act ? t.lane : 0)) * CW;
     t.left = t.lane == 0 ? K::LU - 1 : t.lane - 1;
     t.right = t.lane >= K::LU - 1 ? 0 : t.lane + 1;
     t.par = t.rpar = 0;
     t.mask = 0u;
     double *U = a.buf + smp * as_tile_per_sample(N), *G = U + nn, *W = G + nn;
     // the thread's slot of p, q and d: row y at + y * N * NW floats... [row][warp][lane] vectors
-    const int slot = (t.warp * K::LU + t.lane) * CW;
     constexpr int SROW = K::NW * K::LU * CW;
-    float *D = reinterpret_cast<float *>(W + nn) + slot, *Pp = at_smem + K::P + slot, *Qp = at_smem + K::Q + slot;
+    float *D = reinterpret_cast<float *>(W + nn) + t.slot, *Pp = at_smem + K::P + t.slot, *Qp = at_smem + K::Q + t.slot;
     const int own = t.warp * RW * N + (act ? t.lane : 0) * CW;  // the thread's first point
     if (threadIdx.x <= a.R) widths[threadIdx.x] = a.widths[threadIdx.x];
     const double eps = a.eps ? a.eps[smp] : a.eps_nominal;
@@ -635,7 +677,8 @@ __global__ void __launch_bounds__(AtCfg<N>::NT, MINB) active_set_tile_kernel(con
             }
             const float fmax = (float)fbound;
             if (fmax < FLT_MIN) continue;  // F = 0 with a new active set: the next pass confirms it
-            at_tail_diagonals<N>(t);
+            at_hold_tail<N>(t);
+            if constexpr (K::HOLD) t.template hold_relax<1>();
             const float sc = 1.0f / fmax;  // scaled to max |f| = 1
 #pragma unroll
             for (int y = 0; y < RW; ++y)
