@@ -803,7 +803,7 @@ def run_paper(args):
     if args.beta2 == 0:
         fft_models = [mfmc.Model(n=n, delta=d, algo=mfmc.ALGO_FFT, **common) for n, d in levels]
         fft_cost = [_batched_cost(mfmc, m, 256, base + 10 ** 7) for m in fft_models]
-        # the own-FFT spectral form (register transforms on 64 and 128, mixed-radix on 88)
+        # the own-FFT spectral form (half-lattice transforms on 64, 88 and 128)
         spec_cost = [_batched_cost(mfmc, mfmc.Model(n=n, delta=d, algo=mfmc.ALGO_SPECTRAL, **common), 256,
                                    base + 10 ** 7) for n, d in levels]
     else:

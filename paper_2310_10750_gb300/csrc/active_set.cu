@@ -49,6 +49,8 @@
 namespace mfmc {
 
 constexpr int AS_NT = 512;
+constexpr int AS_NU = 2;              // damped-Jacobi sweeps before and after each coarse correction
+constexpr int AS_NU_COARSE = 16;
 constexpr int AS_VEC64 = 3;           // u, g, w
 constexpr int AS_VEC32 = 7;           // d, r, p, q, inactive mask, z, t
 constexpr int AS_MAX_LEVELS = 8;

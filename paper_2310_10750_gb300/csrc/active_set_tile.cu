@@ -13,14 +13,18 @@
 // and 1 x 4), each level's mask average a population count of the thread's bits, restriction
 // and prolongation exchanging one row per warp.  The levels below one column a lane (16^2 and
 // 8^2, or 11^2 for n = 88) are one warp's work, in its registers.  A pass costs one CTA barrier (the
-// row exchange alternates two buffers), no division and no index arithmetic.
+// row exchange alternates two buffers) and no index arithmetic; the relaxation factors are divided once
+// a Newton pass.  f and v are 32 registers each (n = 64: 16) where the launch allows 128, 80 and 64 a
+// thread, so parts of them spill around the coarse levels (bytes of stores a thread: 128^2 516, 88^2
+// 1456, 64^2 520; L1 holds them).
 //
 // What bounds it: the fallback kernel (fine-level vectors in L2, generic indices) issued 943
 // instructions per point and CG iteration, and waited on L2 (long scoreboard 4.4 cycles an
-// instruction).  Here the FP64 pipe (two lanes a clock an SM) takes the larger part of a step:
-// the disc sum's transforms (444 K cycles a step of 128^2) and 7 operations per point of a Newton
-// residual (88 K); a V-cycle is 21 K cycles.  beta2 = 0.05: 50 samples of 128^2, 20 steps, 17.1 ms
-// (fallback kernel 113), 1000 of 64^2, 10 steps, 11.2 ms (106), 304 of 88^2, 8 steps, 8.4 ms.
+// instruction).  Here the FP64 pipe (two lanes a clock an SM) takes the larger part of a step, 52 % busy
+// over 128^2 solves and 69 % over 64^2: the disc sum's transforms (444 K cycles a step of 128^2) and 7
+// operations per point of a Newton residual (88 K); a V-cycle is 20 K cycles.  beta2 = 0.05: 50
+// samples of 128^2, 20 steps, 17.3 ms (fallback kernel 113), 1000 of 64^2, 10 steps, 11.3 ms (106), 304
+// of 88^2, 8 steps, 8.6 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>

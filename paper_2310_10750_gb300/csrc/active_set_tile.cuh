@@ -9,10 +9,9 @@
 namespace mfmc {
 
 // Constants of the correction solve shared by both kernels.
-constexpr float AS_CG_RTOL = 1e-5f;   // max |J d + F| / max |F| that ends a correction
-constexpr int AS_NU = 2;              // damped-Jacobi sweeps before and after each coarse correction
-constexpr int AS_NU_COARSE = 16;
-constexpr float AS_OMEGA = 0.8f;
+constexpr float AS_CG_RTOL = 1e-5f;   // max |J d + F| / max |F| that ends a correction (active_set_tile.cu:
+                                      // one of its tolerances)
+constexpr float AS_OMEGA = 0.8f;      // damping of the Jacobi sweeps
 
 struct alignas(16) AsFactor {
     double x, y, z, w;  // a row of hf_product_table

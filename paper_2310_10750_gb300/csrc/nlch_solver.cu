@@ -413,7 +413,7 @@ bool algo_supported(const Model &m, int algo) {
     // beta2 > 0: only the active-set solver; it serves nothing else
     if (m.d.beta2 > 0.0 || algo == MFMC_ALGO_ACTIVE_SET) return m.d.beta2 > 0.0 && algo == MFMC_ALGO_ACTIVE_SET;
     if (algo == MFMC_ALGO_FFT) return m.d.bc == MFMC_BC_PERIODIC;  // any kernel, any radius
-    if (algo == MFMC_ALGO_SPECTRAL) return spectral_supported(m);   // any kernel and radius, n = 1024
+    if (algo == MFMC_ALGO_SPECTRAL) return spectral_supported(m);   // any kernel and radius
     if (algo == MFMC_ALGO_WEIGHTED)  // any radial kernel, integer delta / h, either boundary
         return m.integer_R && tma_launcher(m.R) != nullptr && tma_launcher(m.R)->v[kTmaWeighted].fn[3] != nullptr;
     // a non-integer delta / h: only the generic kernel, whose disc is set at run time

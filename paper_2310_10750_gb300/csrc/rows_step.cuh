@@ -472,7 +472,7 @@ RowsLauncher make_rows_launcher() {
     return L;
 }
 
-// Defined in the per-R translation units (R <= 8).
+// The instances of rows_launch.cu (R in {2, 4, 6, 8, 12, 16}), or nullptr.
 const RowsLauncher *rows_launcher(int R);
 
 }  // namespace mfmc

@@ -415,7 +415,9 @@ __device__ __forceinline__ void sq_tile(const SqModelDev &M, int s, float2 *smem
 // model first (the host orders the models), and run each with the fastest form for its lattice.
 // TILE: the launch has tile-form items (n = 64, 88, 128): sixteen warps, of which a 128^2 sample
 // takes all, an 88^2 sample eleven and each half two of a 64^2 item's four samples.  Without them
-// nine warps at fewer registers, two CTAs per SM.
+// nine warps at fewer registers, two CTAs per SM.  (88^2 items alone in the sixteen-warp form, 100
+// steps: 600 samples of three models 2.23 ms, 304 of one 1.13; in the nine-warp mixed-radix form before
+// it 7.77 and 3.91.)
 template <bool TILE>
 __global__ void __launch_bounds__(TILE ? kSqTileThreads : kSqThreads, TILE ? 1 : 2)
     spectral_queue_kernel(const __grid_constant__ SqArgs a) {
@@ -457,12 +459,12 @@ __global__ void __launch_bounds__(TILE ? kSqTileThreads : kSqThreads, TILE ? 1 :
 
 // One sample per CTA (a batch of one tile-form model).
 template <int N, int MINB>
-__global__ void __launch_bounds__(HfCfg<N>::NT, MINB) spectral_tile_kernel(const __grid_constant__ SqModelDev M, int s0,
-                                                                           TraceBuf trace) {
+__global__ void __launch_bounds__(HfCfg<N>::NT, MINB)
+    spectral_tile_kernel(const __grid_constant__ SqModelDev M, TraceBuf trace) {
     extern __shared__ __align__(16) float sq_smem[];
     __shared__ double red[HfCfg<N>::NW];
     const unsigned long long t0 = trace.rec ? trace_clock() : 0ull;
-    const int s = s0 + blockIdx.x;
+    const int s = blockIdx.x;
     sq_tile<N>(M, s, reinterpret_cast<float2 *>(sq_smem), red, 0, 0);
     if (threadIdx.x == 0) trace_put(trace, kTraceSpectralQueue, (uint32_t)s, 0, t0);
 }
@@ -680,7 +682,7 @@ static mfmc_status run_solve_spectral_tile(Model &m, const StepCoef *coef, const
     constexpr size_t smem = hf_smem_bytes<N, float>();
     MFMC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     // (a trace record per sample on n = 88 only, as the trace's description says)
-    kern<<<(unsigned)ns, HfCfg<N>::NT, smem, st>>>(d, 0, N == 88 ? trace_buf() : TraceBuf{});
+    kern<<<(unsigned)ns, HfCfg<N>::NT, smem, st>>>(d, N == 88 ? trace_buf() : TraceBuf{});
     MFMC_LAUNCHED("spectral launch 4");
     return MFMC_OK;
 }

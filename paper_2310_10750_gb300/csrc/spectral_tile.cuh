@@ -5,7 +5,7 @@
 //
 // What bounds it: the FMA pipe and shared memory, about evenly (per 128^2 step 1.26 M FP32
 // operations, 9.8 K cycles at 128 a clock, and 6.1 K cycles of shared-memory traffic on an SM).
-// 100 steps of 256 samples: 128^2 1.32 ms, 88^2 0.74; of 1000 samples of 64^2 1.02.  The forms
+// 100 steps of 256 samples: 128^2 1.28 ms, 88^2 0.75; of 1000 samples of 64^2 1.03.  The forms
 // before it (one complex transform per two rows, split and merged around the product, the field in
 // shared memory; mixed radix at 88): 2.57, 3.21 and 2.34 ms.
 #pragma once

@@ -50,3 +50,20 @@ def test_rows_one_step_against_the_oracle(gpu_lib, n, R):
     torch.cuda.synchronize()
     ref, _ = o.solve(u0[1].cpu().numpy().astype(np.float64), 0.02)
     assert np.abs(uT[1].cpu().numpy() - ref).max() <= 4e-6
+
+
+def test_auto_long_short_long(gpu_lib):
+    # AUTO runs the short batch on the tile kernel, over the scratch that the long ones use plain
+    import torch
+    mf = gpu_lib
+    kw = dict(n=512, delta=16 / 512, eps=0.02, tau=2e-3, ic=2, nsteps=2)
+    auto, tile = mf.Model(**kw), mf.Model(algo=mf.ALGO_PREFIX_TMA, **kw)
+    u0 = torch.empty((45, 512, 512), dtype=torch.float32, device="cuda")
+    mf.mfmc_init_fields(auto, list(range(45)), u0)
+    ref = torch.empty_like(u0)
+    mf.mfmc_solve_fields(tile, u0, 45, uT=ref)
+    for ns in (2, 45, 2, 45, 45):
+        uT = torch.full_like(u0, 7.0)
+        mf.mfmc_solve_fields(auto, u0, ns, uT=uT)
+        torch.cuda.synchronize()
+        assert torch.equal(uT[:ns], ref[:ns]) and bool((uT[ns:] == 7.0).all())
