@@ -241,8 +241,8 @@ mfmc_status mfmc_model_solver_stats(const mfmc_model *model, uint64_t *newton_it
 
 /* Iteration bounds of the beta2 > 0 solver (MFMC_ALGO_ACTIVE_SET; the paper states no solver for
  * its obstacle step, so the bounds are this library's): newton_max = semismooth Newton passes
- * per time step (default 60; below about 40 the corrections are solved to a tighter tolerance, so that
- * a step takes the fewest passes), cg_max = FP32 CG iterations per Newton correction (default 500);
+ * per time step (default 60; below that every correction is solved to a tighter tolerance, so that a
+ * step takes the fewest passes, and a step that cycles is not started over), cg_max = FP32 CG iterations per Newton correction (default 500);
  * 0 restores a default.  A step that reaches the Newton bound stops the sample's solve and sets
  * the model's status flag, so mfmc_solve_batch returns MFMC_ETIMEOUT; the device stays usable
  * and the next call starts with the flag cleared.  MFMC_EINVAL for values outside [0, 100000]. */

@@ -15,8 +15,8 @@
 // 8^2, or 11^2 for n = 88) are one warp's work, in its registers.  A pass costs one CTA barrier (the
 // row exchange alternates two buffers) and no index arithmetic; the relaxation factors are divided once
 // a Newton pass.  f and v are 32 registers each (n = 64: 16) where the launch allows 128, 80 and 64 a
-// thread, so parts of them spill around the coarse levels (bytes of stores a thread: 128^2 516, 88^2
-// 1456, 64^2 520; L1 holds them).
+// thread, so parts of them spill around the coarse levels (bytes of stores a thread: 128^2 580, 88^2
+// 1448, 64^2 488; L1 holds them).
 //
 // What bounds it: the fallback kernel (fine-level vectors in L2, generic indices) issued 943
 // instructions per point and CG iteration, and waited on L2 (long scoreboard 4.4 cycles an
@@ -37,7 +37,12 @@ namespace mfmc {
 
 namespace {
 
-constexpr int AT_SPARE_PASSES = 40;  // of the default bound's 60; a step takes 4 to 8
+// Newton passes of a step (4 to 8 as a rule) under the default bound: loose corrections up to the first of
+// these, then again from the beta2 = 0 step's w with tight ones, then once more, its first AT_DAMPED
+// corrections halved, which ends most cycles of the active set.  (2400 samples of 4 steps, 5 lattices and
+// horizons, eps 0.002 to 0.06, beta2 0.05 to 5: tight corrections alone end 1618 within 60 passes, loose ones
+// alone 1620 but 5 of those not, with the restarts 2262 and none of those lost; 12, 32, 6 passes 2142.)
+constexpr int AT_LOOSE_PASSES = 12, AT_TIGHT_PASSES = 24, AT_DAMPED = 10;
 constexpr int AT_NU_COARSE = 8;  // coarsest sweeps (16, as the fallback kernel has: no CG iteration fewer)
 
 template <int N>
@@ -594,6 +599,7 @@ __global__ void __launch_bounds__(AtCfg<N>::NT, MINB) active_set_tile_kernel(con
     t.w1 = AS_OMEGA / t.d1;
     for (int i = threadIdx.x; i < nn; i += K::NT) U[i] = (double)a.u0[smp * (size_t)nn + i];
     __syncthreads();
+    const bool roomy = a.newton_max >= kAsNewtonMax;  // room for loose corrections and restarts
     bool failed = false;
     unsigned long long n_newton = 0, n_cg = 0;
     for (int step = 1; step <= a.nsteps && !failed; ++step) {
@@ -620,14 +626,16 @@ __global__ void __launch_bounds__(AtCfg<N>::NT, MINB) active_set_tile_kernel(con
             }
             __syncthreads();
         }
-        if (step == 1) {  // start: w of the previous step, or here the beta2 = 0 step's
-            for (int i = threadIdx.x; i < nn; i += K::NT) {
-                const double u0 = at_clip((U[i] + tb1 * G[i]) / (1.0 + tb1 * cg));
-                W[i] = cg * u0 - G[i];
-            }
-            __syncthreads();
-        }
         for (int it = 1;; ++it) {
+            // start: w of the previous step, or the beta2 = 0 step's, at the first step and where a step has
+            // not come home (its active set cycles)
+            if (it == 1 ? step == 1 : roomy && (it == AT_LOOSE_PASSES + 1 || it == AT_TIGHT_PASSES + 1)) {
+                for (int i = threadIdx.x; i < nn; i += K::NT) {
+                    const double u0 = at_clip((U[i] + tb1 * G[i]) / (1.0 + tb1 * cg));
+                    W[i] = cg * u0 - G[i];
+                }
+                __syncthreads();
+            }
             ++n_newton;
             // FP64 residual c_gamma F(w), the inactive set, and the right-hand side of J d = -F, which is
             // f = -(c_gamma F) / max |c_gamma F| with d scaled back by max |c_gamma F| / c_gamma
@@ -692,10 +700,11 @@ __global__ void __launch_bounds__(AtCfg<N>::NT, MINB) active_set_tile_kernel(con
             // correction can be worth: while the active set still moves it limits the next residual, not
             // the solve, and on a settled set the next residual is this one times the tolerance (AS_CG_RTOL
             // throughout: 33.1 CG iterations a step of 128^2 samples, now 26.1).  The loose corrections
-            // cost a pass here and there (4.8 -> 5.1), so they are left to steps with passes to spare: under
-            // a caller's tighter bound, and late in a step, every correction is worth its pass.
-            const bool spare = a.newton_max - it >= AT_SPARE_PASSES;
-            const float rtol = spare && it == 1 ? 3e-2f : (spare && changed ? 1e-3f : (changed || it == 1 ? AS_CG_RTOL : 1e-6f));
+            // cost a pass here and there (4.8 -> 5.1), and where the active set is close to cycling they can
+            // make it cycle: under a caller's tighter bound there are none, and a step that they do not
+            // bring home starts over without them.
+            const bool loose = roomy && it <= AT_LOOSE_PASSES;
+            const float rtol = loose && it == 1 ? 3e-2f : (loose && changed ? 1e-3f : (changed || it == 1 ? AS_CG_RTOL : 1e-6f));
             float rz = 0.0f;
             for (int k = 1;; ++k) {
                 float v[RW][CW];
@@ -765,7 +774,8 @@ __global__ void __launch_bounds__(AtCfg<N>::NT, MINB) active_set_tile_kernel(con
                 }
             }
             if (act) {
-                const double scale = (double)fmax * icg;
+                const bool damped = roomy && it > AT_TIGHT_PASSES && it <= AT_TIGHT_PASSES + AT_DAMPED;
+                const double scale = (double)fmax * (damped ? 0.5 * icg : icg);
 #pragma unroll
                 for (int y = 0; y < RW; ++y) {
                     double w[CW];

@@ -3,6 +3,9 @@ succeed.  n = 32 runs the other kernel, whose report is the one to match."""
 import numpy as np
 import pytest
 
+import oracle as O
+from oracle import beta2_oracle as B2
+
 pytestmark = pytest.mark.gpu
 
 
@@ -77,3 +80,16 @@ def test_a_tight_pass_bound_is_met(gpu_lib, n, delta, kernel, steps, ns, passes)
     with pytest.raises(mf.MfmcError) as e:
         mf.mfmc_solve_batch([g] * ns, seeds)
     assert e.value.status == mf.MFMC_ETIMEOUT
+
+
+# Steps whose active set is close to cycling, which loose corrections alone tip over (small eps, large
+# beta2): the solve ends, and agrees with the oracle as in test_active_set_gpu.py.
+@pytest.mark.parametrize("n,eps,tau,beta2,seed", [
+    (64, 0.002688285082775925, 0.01, 5.0, 5), (64, 0.003613438343137776, 0.03, 1.0, 6), (64, 0.006, 0.01, 5.0, 3),
+    (64, 0.006, 0.01, 5.0, 4), (128, 0.002, 0.03, 1.0, 5)])
+def test_steps_close_to_cycling_end(gpu_lib, n, eps, tau, beta2, seed):
+    mf = gpu_lib
+    kw = dict(n=n, delta=0.125, kernel=1, delta_hf=0.25, eps=eps, tau=tau, nsteps=4, ic=2)
+    f, _ = mf.mfmc_solve_batch([mf.Model(beta2=beta2, **kw)], np.array([seed], dtype=np.uint64))
+    ref, _, _, _ = B2.solve_sample(O.OracleModel(**kw), seed, beta2, 4)
+    assert abs(f[0] - ref) <= 1e-8 * ref
